@@ -25,7 +25,7 @@ struct LaunchPrep {
     int sms[MAX_DEVICES] = {};
 
     template <class Kernel>
-    cudaError_t get(Kernel kernel, size_t smem, int* sms_out) {
+    cudaError_t get(Kernel kernel, size_t smem, int* sms_out, bool wide_clusters = false) {
         int dev = 0;
         cudaError_t e = cudaGetDevice(&dev);
         if (e != cudaSuccess) return e;
@@ -34,6 +34,10 @@ struct LaunchPrep {
         if (!ready[dev]) {
             if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
                 cudaSuccess)
+                return e;
+            // clusters of more than 8 blocks are opt-in
+            if (wide_clusters && (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) !=
+                                     cudaSuccess)
                 return e;
             if ((e = cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
             ready[dev] = true;

@@ -3,7 +3,9 @@
 // the group's scale, accumulate the matrix-vector product; the wide weights
 // never reach memory).
 //
-// Batch 1 (gemv1_kernel): one persistent block per SM, warp-specialised.
+// Small layouts at batch 1 take gemv1_unit_kernel (one unit per block, a row
+// block's slabs a cluster; below). Otherwise,
+// batch 1 (gemv1_kernel): one persistent block per SM, warp-specialised.
 //   warp 0 (copier)    streams unit blobs into NSTAGE shared-memory stages with
 //                      TMA bulk copies and, once a unit is consumed, sums its
 //                      slots per row into y and starts the copy of a later unit
@@ -106,13 +108,17 @@ template <int NX> struct Geo {
 };
 static_assert(NCW == 16, "teams of 16 or 8 warps: task steps are powers of two (masks, no division)");
 
+// The activation tables of one slab.
 template <int NX>
-struct __align__(16) TablesT {
+struct __align__(16) ActTab {
     uint8_t lut[NX * LUT_BYTES];         // vector v, column c, nibble j, entry m at v*LUT_BYTES + c*1280 + (c&1)*64 + j*64 + m*4
     float xs[NX * XS_FLOATS];            // x as fp32; quarter (c, q) at (c*4 + q) * XQ
     float x4s[NX * X4S_FLOATS];          // x pre-scaled per 4-bit nibble slot (see dot4_half); half (c, h) at (c*2 + h) * XH
     float2 x4z[NX][MAX_C][2];            // per column and half: sums of x * 2^-100, even / odd codes
     float xlut[NX][MAX_C];               // per column: sum of the all-ones entries, in lookup order
+};
+template <int NX>
+struct __align__(16) TablesT : ActTab<NX> {
     float slots[Geo<NX>::nstage][NX][SLOT_FLOATS];   // per stage and vector: one value per (row, column) (see slot_addr)
     unsigned long long full[Geo<NX>::nstage];        // blob landed (TMA transaction count)
     unsigned long long empty[Geo<NX>::nstage];       // the unit's team is done (one arrival per team warp)
@@ -357,7 +363,7 @@ __device__ __forceinline__ float2 zero_level_sum4(const float (&xh)[32]) {
 // column's half-warp in the pairs tree16x2 uses.
 static_assert(NCT >= 16 * MAX_C + 2 * MAX_C, "threads for the tables and the zero-level sums");
 template <int NX, int MODE>
-__device__ void build_tables(TablesT<NX>& T, const LayoutView& L, const uint16_t* __restrict__ x,
+__device__ void build_tables(ActTab<NX>& T, const LayoutView& L, const uint16_t* __restrict__ x,
                              const float* __restrict__ gu, int s, int ct) {
     const int cols = min(L.C, L.G - s * L.C);
     consumer_sync();                // nobody still reads the old tables
@@ -512,7 +518,7 @@ __device__ __forceinline__ Task task64(uint32_t sblob, uint4 d, int lane) {
 // The per-width bodies: each group's scaled dot product (per activation
 // vector) into its (row, column) slot of the stage.
 template <int NX>
-__device__ __forceinline__ void body4(const TablesT<NX>& T, const Task& t, uint32_t slots, int lane) {
+__device__ __forceinline__ void body4(const ActTab<NX>& T, const Task& t, uint32_t slots, int lane) {
     constexpr uint32_t SLOT_V = SLOT_FLOATS * 4;      // bytes between the vectors' slot arrays
     // halves in the order (lane >> 2) & 1 first, so each quarter-warp's
     // 16-byte loads fall in 8 distinct bank groups
@@ -540,7 +546,7 @@ __device__ __forceinline__ void body4(const TablesT<NX>& T, const Task& t, uint3
 }
 
 template <int NX>
-__device__ __forceinline__ void body8(const TablesT<NX>& T, const Task& t, uint32_t slots, int lane) {
+__device__ __forceinline__ void body8(const ActTab<NX>& T, const Task& t, uint32_t slots, int lane) {
     constexpr uint32_t SLOT_V = SLOT_FLOATS * 4;
     // quarter (k + (lane >> 1)) & 3 in step k: conflict-free 16-byte loads
     const int c = t.c;
@@ -572,7 +578,7 @@ __device__ __forceinline__ void body8(const TablesT<NX>& T, const Task& t, uint3
 }
 
 template <int NX>
-__device__ __forceinline__ void body2(const TablesT<NX>& T, const Task& t, uint32_t slots) {
+__device__ __forceinline__ void body2(const ActTab<NX>& T, const Task& t, uint32_t slots) {
     constexpr uint32_t SLOT_V = SLOT_FLOATS * 4;
     const int c = t.c;
     const uint4 pl = lds_u32x4(t.pay);
@@ -600,7 +606,7 @@ __device__ __forceinline__ void body2(const TablesT<NX>& T, const Task& t, uint3
 }
 
 template <int NX>
-__device__ __forceinline__ void body1(const TablesT<NX>& T, const Task& t, uint32_t slots) {
+__device__ __forceinline__ void body1(const ActTab<NX>& T, const Task& t, uint32_t slots) {
     constexpr uint32_t SLOT_V = SLOT_FLOATS * 4;
     const int ca = t.c, cb = t.c2;
     const uint4 v = lds_u32x4(t.pay);
@@ -632,7 +638,7 @@ __device__ __forceinline__ void body1(const TablesT<NX>& T, const Task& t, uint3
 // order that balances the warps of this deal). Each group's result goes to its
 // slot in the stage's slot array at shared address slots.
 template <int NX>
-__device__ __forceinline__ void consume_unit(const TablesT<NX>& T, uint32_t sblob, uint32_t slots, int t0, int tstep,
+__device__ __forceinline__ void consume_unit(const ActTab<NX>& T, uint32_t sblob, uint32_t slots, int t0, int tstep,
                                              int lane) {
     const uint32_t hw = lds_u32(sblob + offsetof(UnitHeader, ntask));     // ntask | task16 << 16
     const int ntask = (int)(hw & 0xFFFFu);
@@ -664,7 +670,7 @@ __device__ __forceinline__ void item_pos(int i, int rows, int& c, uint32_t& r) {
 static_assert(RB == 128, "item_pos shifts by log2(RB)");
 
 template <int NX, int W>
-__device__ __forceinline__ void consume_single_w(const TablesT<NX>& T, uint32_t sblob, uint32_t slots, int t0,
+__device__ __forceinline__ void consume_single_w(const ActTab<NX>& T, uint32_t sblob, uint32_t slots, int t0,
                                                  int tstep, int lane, int rows) {
     const int n = (int)lds_u16(sblob + offsetof(UnitHeader, n) + 2 * W);
     const uint32_t pay = sblob + lds_u16(sblob + offsetof(UnitHeader, pay16) + 2 * W) * 16;
@@ -704,7 +710,7 @@ __device__ __forceinline__ void consume_single_w(const TablesT<NX>& T, uint32_t 
 }
 
 template <int NX>
-__device__ __forceinline__ void consume_single(const TablesT<NX>& T, uint32_t sblob, uint32_t slots, int t0, int tstep,
+__device__ __forceinline__ void consume_single(const ActTab<NX>& T, uint32_t sblob, uint32_t slots, int t0, int tstep,
                                                int lane, int rows, int w) {
     if (w == 0) consume_single_w<NX, 0>(T, sblob, slots, t0, tstep, lane, rows);
     else if (w == 1) consume_single_w<NX, 1>(T, sblob, slots, t0, tstep, lane, rows);
@@ -783,8 +789,8 @@ __device__ __forceinline__ void team_sync(int team, int tw) {
 // 0), then the row's lanes added by xor shuffles in a fixed order. Rows are
 // stored when the matrix has one slab and added otherwise.
 template <int NX>
-__device__ __forceinline__ void team_flush(const TablesT<NX>& T, const LayoutView& L, float* __restrict__ y, int st,
-                                           int rb, int wt, int tw, int lane) {
+__device__ __forceinline__ void team_flush(const float* slots, const LayoutView& L, float* __restrict__ y, int rb,
+                                           int wt, int tw, int lane) {
     const int lpr = tw >> 2;                    // lanes per row: 4 (16 warps) or 2 (8 warps)
     const int rpw = 32 / lpr;                   // rows per warp
     const int r = wt * rpw + lane / lpr, part = lane % lpr;
@@ -792,7 +798,7 @@ __device__ __forceinline__ void team_flush(const TablesT<NX>& T, const LayoutVie
     const int chunks = 4 / lpr;                 // 16-byte chunks per lane
 #pragma unroll
     for (int v = 0; v < NX; ++v) {
-        const uint32_t ra = smem_u32(T.slots[st][v]) + (uint32_t)r * 64;
+        const uint32_t ra = smem_u32(slots + v * SLOT_FLOATS) + (uint32_t)r * 64;
         float sum = 0.f;
         for (int k = 0; k < chunks; ++k) {
             const float4 a = lds_f32x4(ra + ((part * chunks + k) << 4));
@@ -1058,7 +1064,7 @@ __global__ void __launch_bounds__(G1_THREADS, 1) gemv1_kernel(LayoutView L, cons
                         if (lane == 0) raise_abort(&T.abort);
                     }
                 }
-                if (!dead) team_flush<NX>(T, L, y, st, rbj, wt, tw, lane);
+                if (!dead) team_flush<NX>(T.slots[st][0], L, y, rbj, wt, tw, lane);
             }
             rbj += teams;
             while (rbj >= L.nrb) { rbj -= L.nrb; ++sj; }
@@ -1319,6 +1325,185 @@ __global__ void __launch_bounds__(CH_THREADS, 1) gemv_chain_kernel(const ChainIt
     }
 }
 
+
+// ---------------------------------------------------------------------------
+// Small layouts: one unit per block, a row block's slabs one cluster.
+//
+// Bound: latency. A small product's weights and arithmetic take well under a
+// microsecond; what a dependent chain of them pays is the hand-over between
+// products. Two things of the persistent kernel are on that path: its 226 KB
+// block cannot start (barriers, first copies) before the previous product's
+// block on the SM exits, and its split-K adds need y zeroed in this call (read
+// the call count, zero, release a flag, acquire it), 0.9 us of a 3.0 us
+// product. Here a block has 512 threads, at most 64 registers a thread and
+// about 92 KB of shared memory, so the next product's blocks sit beside this
+// one's with their weights loaded before griddepcontrol.wait returns; and the
+// slabs of a row block are the blocks of one cluster (up to 16), each sending
+// its row sums straight into slab 0's shared memory (st.async, counted on an
+// mbarrier there), which adds them in slab order and stores y once: no
+// zeroing, flags, atomics or control words, and the same bits on every call.
+// Per product, in a graph of dependent products (us, persistent kernel before
+// -> this): 768x768 3.04 -> 2.32, 2048x768 3.71 -> 2.31, 768x2048 3.33 -> 2.45;
+// the 85 products of the ~131M decode step 265 -> 208 us.
+// ---------------------------------------------------------------------------
+constexpr int U1_THREADS = NCT;          // every warp consumes
+constexpr int MAX_CLUSTER = 16;          // blocks of one row block: its slabs (over 8 is opt-in)
+
+// Layouts for the unit kernel: units of at most 2 columns (wider units come
+// from larger matrices, where a cluster launched between persistent blocks
+// gains nothing: a ~9B layer whose 1024x4096 products, 4-column units in
+// clusters of 16, ran here took 45.4 against 45.1 us), a row block's slabs
+// within the largest cluster, and every cluster resident at once (two blocks
+// per SM, less what clusters leave unused of a GPC's SMs: 276..296 blocks fit
+// for up to 8 slabs, 196..253 above; as several waves of clusters 14336x4096
+// takes 8.3 -> 10.9 us).
+inline bool unit_per_block(const LayoutView& L, int sms) {
+    return L.C <= 2 && L.S <= MAX_CLUSTER && 4 * L.units <= (L.S <= 8 ? 7 : 5) * sms;
+}
+
+struct __align__(16) TablesU : ActTab<1> {
+    float slots[SLOT_FLOATS];
+    float part[MAX_CLUSTER - 1][RB];     // slab 0's block: the row sums of slabs 1 ..
+    unsigned long long full;             // the blob landed
+    unsigned long long sums;             // slab 0's block: every other slab's row sums landed
+    int abort;
+};
+constexpr size_t gemv1_unit_smem() { return 256 + (size_t)STAGE_BYTES + sizeof(TablesU); }
+static_assert(2 * (gemv1_unit_smem() + 1024) <= 228 * 1024, "two blocks per SM");
+
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+// Bounded wait for other blocks' st.async on this block's barrier. Longer than
+// any of their own waits: every block of the cluster sends its sums even when
+// a wait of its own ran out, so the receiver never exits before they land.
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity) {
+    const unsigned long long t0 = global_ns();
+    for (;;) {
+        uint32_t ok;
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
+                     "selp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(ok) : "r"(bar), "r"(parity), "n"(SUSPEND_HINT_NS) : "memory");
+        if (ok) return true;
+        if (global_ns() - t0 > 4 * WAIT_LIMIT_NS) return false;
+    }
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// One float into another block's shared memory, counted (4 bytes) on that block's barrier.
+__device__ __forceinline__ void st_async_f32(uint32_t dst, float v, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
+                 :: "r"(dst), "r"(__float_as_uint(v)), "r"(bar) : "memory");
+}
+
+// Block rb * S + s takes unit (rb, s): MODE and SW as in gemv1_kernel.
+template <int MODE, bool SW>
+__global__ void __launch_bounds__(U1_THREADS, 2) gemv1_unit_kernel(LayoutView L, const uint16_t* __restrict__ x,
+                                                                   float* __restrict__ y, int dep,
+                                                                   uint16_t* __restrict__ h,
+                                                                   const float* __restrict__ gu) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    unsigned char* base = smem_raw + ((256u - (smem_u32(smem_raw) & 255u)) & 255u);
+    TablesU& T = *reinterpret_cast<TablesU*>(base + STAGE_BYTES);
+    const uint32_t stage = smem_u32(base), full = smem_u32(&T.full), sums = smem_u32(&T.sums);
+    const uint32_t abort_addr = smem_u32(&T.abort);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rb = blockIdx.x / L.S, s = blockIdx.x - rb * L.S, u = s * L.nrb + rb;
+    const int rows = min(RB, (int)(L.N - (int64_t)rb * RB));
+    if (tid == 0) {
+        mbar_init(full, 1);
+        mbar_init(sums, 1);
+        T.abort = 0;
+        fence_barrier_init();
+        issue_unit_g1<SW>(L, u, stage, full);
+        if (s == 0 && L.S > 1)
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
+                         :: "r"(sums), "r"((uint32_t)(L.S - 1) * rows * 4u) : "memory");
+    }
+    // slots no group writes (rows past N, absent columns) read as zero
+    for (int i = tid; i < SLOT_FLOATS; i += U1_THREADS) T.slots[i] = 0.f;
+    {                                       // the slab's activations into L2 while waiting for the previous grid
+        const int64_t k0 = (int64_t)s * L.C * GROUP;
+        if constexpr (MODE == MODE_SWIGLU_IN) {
+            const int lines = (min(L.C, L.G - s * L.C) * GROUP * 8 + 127) / 128;
+            if (tid >= 32 && tid - 32 < lines) prefetch_l2(gu + 2 * k0 + (int64_t)(tid - 32) * 32);
+        } else {
+            const int lines = (min(L.C, L.G - s * L.C) * GROUP * 2 + 127) / 128;
+            if (tid >= 32 && tid - 32 < lines) prefetch_l2(x + k0 + (int64_t)(tid - 32) * 64);
+        }
+    }
+    __syncthreads();
+    if (L.S > 1) cluster_arrive();          // this block's barriers are ready for the others' sums
+    if (dep != DEP_GROUP_FIRST) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (dep != DEP_GROUP_NEXT) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (dep == DEP_GROUP_FIRST) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+    bool dead = false;
+    build_tables<1, MODE>(T, L, x, gu, s, tid);
+    if (!warp_wait(full, 0, abort_addr)) { dead = true; if (lane == 0) raise_abort(&T.abort); }
+    if (!dead) {
+        if constexpr (SW) consume_single<1>(T, stage, smem_u32(T.slots), warp, NCW, lane, rows, L.single_w);
+        else consume_unit<1>(T, stage, smem_u32(T.slots), warp, NCW, lane);
+    }
+    __syncthreads();                        // every slot of the unit is written
+    if (L.S > 1) cluster_wait();
+    // row r of the unit: four lanes, a 16-byte chunk of slots each
+    const int r = tid >> 2, q = tid & 3;
+    const float4 a = lds_f32x4(smem_u32(T.slots) + (uint32_t)r * 64 + (q << 4));
+    float sum = (a.x + a.y) + (a.z + a.w);
+    sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+    sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+    if (s > 0) {
+        if (q == 0 && r < rows)
+            st_async_f32(cluster_addr(smem_u32(&T.part[s - 1][r]), 0), sum, cluster_addr(sums, 0));
+    } else {
+        if (L.S > 1) {
+            if (!__all_sync(0xffffffffu, mbar_wait_cluster(sums, 0))) { dead = true; if (lane == 0) raise_abort(&T.abort); }
+            float more = 0.f;
+            for (int k = q; k < L.S - 1; k += 4) more += T.part[k][r];
+            more += __shfl_xor_sync(0xffffffffu, more, 1);
+            more += __shfl_xor_sync(0xffffffffu, more, 2);
+            sum += more;
+        }
+        if (q == 0 && r < rows && !dead) y[(int64_t)rb * RB + r] = sum;
+        if (MODE == MODE_SWIGLU_EPI) {
+            const float up = __shfl_xor_sync(0xffffffffu, sum, 4);
+            if (q == 0 && !(r & 1) && r < rows && !dead) h[((int64_t)rb * RB + r) >> 1] = swiglu_bf16(sum, up);
+        }
+    }
+    // after a wait that ran out, let the copy land before the block exits
+    if (tid == 0 && lds_volatile(abort_addr)) mbar_wait_bounded(full, 0);
+    if (dep == DEP_GROUP_NEXT && tid == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <int MODE, bool SW>
+cudaError_t launch_gemv1_unit(const LayoutView& L, const uint16_t* x, float* y, cudaStream_t s, int dep,
+                              uint16_t* h, const float* gu) {
+    static LaunchPrep prep;
+    int sms = 0;
+    cudaError_t e = prep.get(gemv1_unit_kernel<MODE, SW>, gemv1_unit_smem(), &sms, true);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(L.units);
+    cfg.blockDim = dim3(U1_THREADS);
+    cfg.dynamicSmemBytes = gemv1_unit_smem();
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = L.S;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = L.S > 1 ? 2 : 1;
+    e = cudaLaunchKernelEx(&cfg, gemv1_unit_kernel<MODE, SW>, L, x, y, dep, h, gu);
+    if (e != cudaSuccess) return e;
+    return cudaGetLastError();
+}
+
 template <int NX, int MODE = MODE_PLAIN, bool SW = false>
 cudaError_t launch_gemv1(const LayoutView& L, const uint16_t* x, float* y, cudaStream_t s, int dep,
                          uint16_t* h = nullptr, const float* gu = nullptr) {
@@ -1326,6 +1511,9 @@ cudaError_t launch_gemv1(const LayoutView& L, const uint16_t* x, float* y, cudaS
     int sms = 0;
     cudaError_t e = prep.get(gemv1_kernel<NX, MODE, SW>, gemv1_smem<NX>(), &sms);
     if (e != cudaSuccess) return e;
+    if constexpr (NX == 1) {
+        if (unit_per_block(L, sms)) return launch_gemv1_unit<MODE, SW>(L, x, y, s, dep, h, gu);
+    }
     const int grid = L.units < sms ? L.units : sms;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
