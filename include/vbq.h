@@ -91,7 +91,7 @@ typedef struct vbq_layout vbq_layout;
  * So codes and scales are a pure function of w and the widths. The call
  * validates widths and NaNs on the device first and synchronises `stream`
  * (outputs are untouched on an error), then enqueues the quantisation and
- * returns without waiting. It allocates a 4-byte temporary.
+ * returns without waiting. It allocates nothing on the device.
  */
 vbq_status_t vbq_quantize(const float* w, const uint8_t* bitwidths, int64_t N, int64_t K,
                           uint8_t* codes_out, uint16_t* scales_out, void* stream);

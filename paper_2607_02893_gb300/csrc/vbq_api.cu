@@ -5,6 +5,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <vector>
 
 #include "../../include/vbq.h"
@@ -41,7 +42,9 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 
 size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-// Device buffers that vbq_pack frees on every exit path.
+// Device buffers that vbq_pack frees on every exit path. (Plain allocations: a
+// small one costs 2-5 us, a stream-ordered one about 50 us and as much again
+// when the next synchronisation trims its pool, measured on a GB300 host.)
 struct TempBuffers {
     std::vector<void*> ptrs;
     ~TempBuffers() {
@@ -53,6 +56,60 @@ struct TempBuffers {
         return e;
     }
 };
+
+// Two error words of one call, in pinned host memory that every device can
+// write: a validating kernel stores to them only on an error, and the host
+// reads them once it has synchronised, without a copy or an allocation per
+// call. The words come from one page shared by all threads (64 calls at a
+// time, one 64-byte line each, given back when the call ends); a call beyond
+// those allocates its own.
+class ErrorWords {
+public:
+    ~ErrorWords() {
+        if (slot_ >= 0) {
+            std::lock_guard<std::mutex> lock(mu_);
+            used_ &= ~(1ull << slot_);
+        } else if (w_) {
+            cudaFreeHost(w_);
+        }
+    }
+    cudaError_t get() {
+        {
+            std::lock_guard<std::mutex> lock(mu_);
+            if (!page_) {
+                const cudaError_t e = host_words(&page_, 4096);
+                if (e != cudaSuccess) return e;
+            }
+            for (int i = 0; i < 64 && slot_ < 0; ++i)
+                if (!(used_ >> i & 1)) slot_ = i;
+            if (slot_ >= 0) {
+                used_ |= 1ull << slot_;
+                w_ = page_ + 16 * slot_;
+            }
+        }
+        if (!w_) {
+            const cudaError_t e = host_words(&w_, 64);
+            if (e != cudaSuccess) return e;
+        }
+        w_[0] = w_[1] = 0;
+        return cudaSuccess;
+    }
+    uint32_t* word(int i) const { return w_ + i; }
+    bool set(int i) const { return static_cast<volatile uint32_t*>(w_)[i] != 0; }
+
+private:
+    static cudaError_t host_words(uint32_t** p, size_t bytes) {
+        return cudaHostAlloc(reinterpret_cast<void**>(p), bytes, cudaHostAllocPortable | cudaHostAllocMapped);
+    }
+    static std::mutex mu_;
+    static uint32_t* page_;
+    static uint64_t used_;
+    uint32_t* w_ = nullptr;
+    int slot_ = -1;
+};
+std::mutex ErrorWords::mu_;
+uint32_t* ErrorWords::page_ = nullptr;
+uint64_t ErrorWords::used_ = 0;
 
 #define VBQ_CUDA(call)                                                                     \
     do {                                                                                   \
@@ -126,6 +183,8 @@ vbq_status_t vbq_pack(const uint8_t* codes, const uint8_t* bitwidths, const uint
     const int64_t G = K / vbq::GROUP;
     const size_t ncodes = (size_t)N * (size_t)K, ngroups = (size_t)N * (size_t)G;
     TempBuffers tmp;
+    ErrorWords err;
+    VBQ_CUDA(err.get());
 
     const uint8_t* d_codes = codes;
     const uint8_t* d_widths = bitwidths;
@@ -143,18 +202,7 @@ vbq_status_t vbq_pack(const uint8_t* codes, const uint8_t* bitwidths, const uint
         d_scales = static_cast<uint16_t*>(ps);
     }
 
-    // 1. validation on the device
-    void* d_err;
-    VBQ_CUDA(tmp.alloc(&d_err, sizeof(uint32_t)));
-    VBQ_CUDA(cudaMemsetAsync(d_err, 0, sizeof(uint32_t), s));
-    VBQ_CUDA(vbq::launch_validate(d_codes, d_widths, N, K, static_cast<uint32_t*>(d_err), s));
-    uint32_t h_err = 0;
-    VBQ_CUDA(cudaMemcpyAsync(&h_err, d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-    VBQ_CUDA(cudaStreamSynchronize(s));
-    if (h_err & 1u) return fail(VBQ_ERR_WIDTH, "a bit-width is not in {1,2,4,8}");
-    if (h_err & 2u) return fail(VBQ_ERR_CODE_RANGE, "a code is >= 2^b for its group's width");
-
-    // 2. plan: row blocks x slabs. Take the widest slab (C in 16..1) that gives
+    // 1. plan: row blocks x slabs (the counting kernel also checks the widths). Take the widest slab (C in 16..1) that gives
     // at least half as many units as SMs and whose largest unit blob fits a
     // stage. (Wider units cost less per group than the imbalance they leave:
     // measured on 1B- and 9B-class shapes, 4096^2 takes 5.8 us with C = 16
@@ -163,8 +211,8 @@ vbq_status_t vbq_pack(const uint8_t* codes, const uint8_t* bitwidths, const uint
     VBQ_CUDA(cudaGetDevice(&dev));
     VBQ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const int64_t nrb = (N + vbq::RB - 1) / vbq::RB;
-    std::vector<uint32_t> counts;
-    std::vector<vbq::UnitHeader> headers;
+    std::vector<uint32_t> counts, sizes;
+    uint32_t* d_counts = nullptr;       // of the chosen plan
     int C = 0;
     int64_t S = 0, units = 0;
     uint32_t max16 = 0;
@@ -175,22 +223,25 @@ vbq_status_t vbq_pack(const uint8_t* codes, const uint8_t* bitwidths, const uint
         if (!last && 2 * uc < sms) continue;          // fewer units than half the SMs: narrower slabs
         if (uc > (1LL << 31) - 2) return fail(VBQ_ERR_UNSUPPORTED, "too many units");
         void* dc = nullptr;
-        VBQ_CUDA(tmp.alloc(&dc, (size_t)uc * 5 * sizeof(uint32_t)));
-        VBQ_CUDA(vbq::launch_count(d_widths, N, (int)G, cand, (int)nrb, (int)uc, static_cast<uint32_t*>(dc), s));
         std::vector<uint32_t> cnt((size_t)uc * 5);
+        VBQ_CUDA(tmp.alloc(&dc, cnt.size() * sizeof(uint32_t)));
+        d_counts = static_cast<uint32_t*>(dc);
+        VBQ_CUDA(vbq::launch_count(d_widths, N, (int)G, cand, (int)nrb, (int)uc, d_counts, err.word(0), s));
         VBQ_CUDA(cudaMemcpyAsync(cnt.data(), dc, cnt.size() * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
         VBQ_CUDA(cudaStreamSynchronize(s));
-        std::vector<vbq::UnitHeader> hd((size_t)uc);
+        if (err.set(0)) return fail(VBQ_ERR_WIDTH, "a bit-width is not in {1,2,4,8}");
+        std::vector<uint32_t> size16((size_t)uc);
         uint32_t m16 = 0;
         for (int64_t u = 0; u < uc; ++u) {
-            hd[u] = vbq::make_header(&cnt[u * 5], cand, (int)cnt[u * 5 + 4]);
-            m16 = std::max<uint32_t>(m16, hd[u].size16);
+            const uint32_t* n = &cnt[u * 5];
+            size16[u] = vbq::make_header(n, cand, (int)n[4]).size16;
+            m16 = std::max<uint32_t>(m16, size16[u]);
         }
         if (m16 * 16u > vbq::MAX_BLOB_BYTES && !last) continue;
         if (m16 * 16u > vbq::MAX_BLOB_BYTES) return fail(VBQ_ERR_UNSUPPORTED, "unit blob too large");
         C = cand; S = Sc; units = uc; max16 = m16;
         counts.swap(cnt);
-        headers.swap(hd);
+        sizes.swap(size16);
         break;
     }
     if (C == 0) return fail(VBQ_ERR_UNSUPPORTED, "no slab width fits");
@@ -199,7 +250,7 @@ vbq_status_t vbq_pack(const uint8_t* codes, const uint8_t* bitwidths, const uint
     uint64_t off16 = 0;
     for (int64_t u = 0; u < units; ++u) {
         blob_off[u] = (uint32_t)off16;
-        off16 += headers[u].size16;
+        off16 += sizes[u];
         for (int w = 0; w < 4; ++w) real_items[w] += counts[u * 5 + w];
         if (off16 > 0xffffffffull) return fail(VBQ_ERR_UNSUPPORTED, "layout too large");
     }
@@ -211,17 +262,12 @@ vbq_status_t vbq_pack(const uint8_t* codes, const uint8_t* bitwidths, const uint
     for (int w = 0; w < 4; ++w) payload_bytes += (size_t)real_items[w] * 8 * (1u << w);
     const size_t scale_bytes = (size_t)ngroups * 2;
 
-    // 3. one device allocation: blob area (+ slack), then the blob offsets
+    // 2. one device allocation: blob area (+ slack), then the blob offsets
     const size_t blob_bytes = (size_t)off16 * 16 + 256;
     const size_t off_at = round_up(blob_bytes, 256);
     const size_t ctl_at = round_up(off_at + blob_off.size() * 4, 256);
     // control words: call counter, zeroed-row flags, SwiGLU slab counts
     const size_t alloc_bytes = ctl_at + (2 + 2 * (size_t)nrb) * sizeof(uint32_t);
-    void* d_headers = nullptr;
-    VBQ_CUDA(tmp.alloc(&d_headers, headers.size() * sizeof(vbq::UnitHeader)));
-    VBQ_CUDA(cudaMemcpyAsync(d_headers, headers.data(), headers.size() * sizeof(vbq::UnitHeader),
-                             cudaMemcpyHostToDevice, s));
-
     vbq_layout* L = new (std::nothrow) vbq_layout();
     if (!L) return fail(VBQ_ERR_NOMEM, "host allocation failed");
     cudaError_t e = cudaMalloc(&L->base, alloc_bytes);
@@ -258,14 +304,19 @@ vbq_status_t vbq_pack(const uint8_t* codes, const uint8_t* bitwidths, const uint
         if (real_items[w]) V.single_w = present++ ? -2 : w;
     if (V.single_w < 0) V.single_w = -1;
 
-    if ((e = cudaMemsetAsync(L->base, 0, alloc_bytes, s)) != cudaSuccess) return bail(VBQ_ERR_CUDA, "memset", e);
+    // control words start at zero; the blobs' alignment padding is never used
+    if ((e = cudaMemsetAsync(V.ctl, 0, alloc_bytes - ctl_at, s)) != cudaSuccess) return bail(VBQ_ERR_CUDA, "memset", e);
     if ((e = cudaMemcpyAsync(base + off_at, blob_off.data(), blob_off.size() * 4, cudaMemcpyHostToDevice, s)) !=
         cudaSuccess)
         return bail(VBQ_ERR_CUDA, "offset copy", e);
-    if ((e = vbq::launch_scatter(d_codes, d_widths, d_scales, static_cast<const vbq::UnitHeader*>(d_headers), V,
-                                 base, s)) != cudaSuccess)
+    if ((e = vbq::launch_scatter(d_codes, d_widths, d_scales, d_counts, V, base, err.word(1), s)) != cudaSuccess)
         return bail(VBQ_ERR_CUDA, "scatter launch", e);
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return bail(VBQ_ERR_CUDA, "pack", e);
+    if (err.set(1)) {
+        cudaFree(L->base);
+        delete L;
+        return fail(VBQ_ERR_CODE_RANGE, "a code is >= 2^b for its group's width");
+    }
     *out = L;
     return VBQ_OK;
 }
@@ -299,19 +350,12 @@ vbq_status_t vbq_quantize(const float* w, const uint8_t* bitwidths, int64_t N, i
     if (!aligned16(w) || !aligned16(bitwidths) || !aligned16(codes_out) || !aligned16(scales_out))
         return fail(VBQ_ERR_ALIGN, "device arrays must be 16-byte aligned");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    // the flag word is a stream-ordered allocation (no device-wide sync on free)
-    void* d_err = nullptr;
-    VBQ_CUDA(cudaMallocAsync(&d_err, sizeof(uint32_t), s));
-    uint32_t h_err = 0;
-    cudaError_t e = cudaMemsetAsync(d_err, 0, sizeof(uint32_t), s);
-    if (e == cudaSuccess) e = vbq::launch_quant_validate(w, bitwidths, N, K, static_cast<uint32_t*>(d_err), s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&h_err, d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
-    const cudaError_t ef = cudaFreeAsync(d_err, s);
-    if (e == cudaSuccess) e = ef;
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    VBQ_CUDA(e);
-    if (h_err & 1u) return fail(VBQ_ERR_WIDTH, "a bit-width is not in {1,2,4,8}");
-    if (h_err & 2u) return fail(VBQ_ERR_ARG, "a weight is NaN");
+    ErrorWords err;
+    VBQ_CUDA(err.get());
+    VBQ_CUDA(vbq::launch_quant_validate(w, bitwidths, N, K, err.word(0), s));
+    VBQ_CUDA(cudaStreamSynchronize(s));
+    if (err.set(0)) return fail(VBQ_ERR_WIDTH, "a bit-width is not in {1,2,4,8}");
+    if (err.set(1)) return fail(VBQ_ERR_ARG, "a weight is NaN");
     VBQ_CUDA(vbq::launch_quantize(w, bitwidths, N, K, codes_out, scales_out, s));
     return VBQ_OK;
 }

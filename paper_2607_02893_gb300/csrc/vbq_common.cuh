@@ -95,54 +95,50 @@ constexpr int TASK_SPAN1 = 64;   // items per 1-bit task
 constexpr int TASK_SPAN = 32;    // items per 2-, 4- and 8-bit task
 constexpr int MAX_UNIT_TASKS = 2 * MAX_UNIT_ITEMS / TASK_SPAN;   // a bound the task cuts never exceed
 
-// The tasks of one unit from its column ends ce[w][c] (w = width index, c <
-// cols): widths 8, 4, 2, 1 bit in that order, each cut into spans of at most
-// TASK_SPAN (TASK_SPAN1) items, a span ending early before an item on which
-// more column ends fall than its masks can count. Writes the descriptors when
-// out is not null (h gives the blob offsets) and returns their number.
-__host__ __device__ inline int unit_tasks(const uint16_t (*ce)[MAX_C], int cols, const UnitHeader* h,
-                                          TaskDesc* out) {
-    int nt = 0;
-    for (int w = 3; w >= 0; --w) {
-        const int span = w == 0 ? TASK_SPAN1 : TASK_SPAN, maxm = w == 0 ? 1 : 3;
-        const int n = cols > 0 ? ce[w][cols - 1] : 0;
-        int st = 0;                     // first item of the next task
-        while (st < n) {
-            const int i0 = w == 0 ? (st & ~1) : st, skip = st - i0;
-            int end = i0 + span < n ? i0 + span : n;
-            uint32_t m1 = 0, m2 = 0;
-            int c0 = 0;                 // ends are nondecreasing: c0 = the first column ending after st
-            while (c0 < cols && ce[w][c0] <= st) ++c0;
-            for (int c = c0; c < cols && ce[w][c] < end;) {
-                const int e = ce[w][c], p = e - i0;
-                int mult = 0;
-                while (c < cols && ce[w][c] == e) { ++mult; ++c; }
-                if (mult > maxm) { end = e; break; }
-                if (w == 0) {
-                    if (p & 1) m2 |= 1u << (p >> 1);
-                    else m1 |= 1u << (p >> 1);
-                } else {
-                    if (mult & 1) m1 |= 1u << p;
-                    if (mult & 2) m2 |= 1u << p;
-                }
+// The tasks of one width of a unit from the width's column ends ce[c] (c <
+// cols): spans of at most TASK_SPAN (TASK_SPAN1) items, a span ending early
+// before an item on which more column ends fall than its masks can count.
+// Writes the descriptors when out is not null (h gives the blob offsets) and
+// returns their number. Column positions only move forward, so a width costs
+// its tasks plus its columns.
+__host__ __device__ inline int width_tasks(const uint16_t* ce, int cols, int w, const UnitHeader* h, TaskDesc* out) {
+    const int span = w == 0 ? TASK_SPAN1 : TASK_SPAN, maxm = w == 0 ? 1 : 3;
+    const int n = cols > 0 ? ce[cols - 1] : 0;
+    int nt = 0, c0 = 0;
+    int st = 0;                         // first item of the next task
+    while (st < n) {
+        const int i0 = w == 0 ? (st & ~1) : st, skip = st - i0;
+        int end = i0 + span < n ? i0 + span : n;
+        uint32_t m1 = 0, m2 = 0;
+        while (c0 < cols && ce[c0] <= st) ++c0;      // the first column ending after st
+        for (int c = c0; c < cols && ce[c] < end;) {
+            const int e = ce[c], p = e - i0;
+            int mult = 0;
+            while (c < cols && ce[c] == e) { ++mult; ++c; }
+            if (mult > maxm) { end = e; break; }
+            if (w == 0) {
+                if (p & 1) m2 |= 1u << (p >> 1);
+                else m1 |= 1u << (p >> 1);
+            } else {
+                if (mult & 1) m1 |= 1u << p;
+                if (mult & 2) m2 |= 1u << p;
             }
-            if (out) {
-                const uint32_t b = 1u << w;
-                TaskDesc d;
-                d.x = (uint32_t)(h->sc16[w] * 16 + 2 * i0) | ((uint32_t)c0 << 16) |
-                      ((uint32_t)(end - i0 - 1) << 20) | ((uint32_t)w << 26) | ((uint32_t)skip << 28);
-                d.y = m1;
-                d.z = m2;
-                d.w = (uint32_t)(h->pay16[w] * 16 + 8 * b * i0) | ((uint32_t)(h->row16[w] * 16 + i0) << 16);
-                out[nt] = d;
-            }
-            ++nt;
-            st = end;
         }
+        if (out) {
+            const uint32_t b = 1u << w;
+            TaskDesc d;
+            d.x = (uint32_t)(h->sc16[w] * 16 + 2 * i0) | ((uint32_t)c0 << 16) | ((uint32_t)(end - i0 - 1) << 20) |
+                  ((uint32_t)w << 26) | ((uint32_t)skip << 28);
+            d.y = m1;
+            d.z = m2;
+            d.w = (uint32_t)(h->pay16[w] * 16 + 8 * b * i0) | ((uint32_t)(h->row16[w] * 16 + i0) << 16);
+            out[nt] = d;
+        }
+        ++nt;
+        st = end;
     }
     return nt;
 }
-
 
 struct LayoutView {
     const uint8_t* blobs;       // blob area
@@ -210,91 +206,6 @@ __host__ __device__ inline UnitHeader make_header(const uint32_t n[4], int C, in
     off += (uint32_t)ntask;
     h.size16 = (uint16_t)off;
     return h;
-}
-
-// ---------------------------------------------------------------------------
-// Item formats: pack 64 codes (64 bytes, one per code) into an item, and back.
-// ---------------------------------------------------------------------------
-
-template <int B>
-__device__ __forceinline__ void pack_item(const uint8_t* __restrict__ src, uint8_t* __restrict__ dst) {
-    uint32_t cw[16];
-    const uint4* p = reinterpret_cast<const uint4*>(src);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        uint4 v = p[q];
-        cw[4 * q] = v.x; cw[4 * q + 1] = v.y; cw[4 * q + 2] = v.z; cw[4 * q + 3] = v.w;
-    }
-    auto code = [&](int j) -> uint32_t { return (cw[j >> 2] >> (8 * (j & 3))) & 0xffu; };
-    if (B == 1 || B == 2) {
-        uint64_t plane[2] = {0, 0};
-#pragma unroll
-        for (int j = 0; j < GROUP; ++j) {
-            const uint64_t c = code(j);
-            plane[0] |= (c & 1ull) << j;
-            if (B == 2) plane[1] |= ((c >> 1) & 1ull) << j;
-        }
-        if (B == 1) {
-            *reinterpret_cast<uint2*>(dst) = make_uint2((uint32_t)plane[0], (uint32_t)(plane[0] >> 32));
-        } else {
-            *reinterpret_cast<uint4*>(dst) = make_uint4((uint32_t)plane[0], (uint32_t)(plane[0] >> 32),
-                                                        (uint32_t)plane[1], (uint32_t)(plane[1] >> 32));
-        }
-    } else if (B == 4) {
-        uint32_t o[8];
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-            uint32_t w = 0;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) w |= code(8 * t + i) << (4 * i);
-            o[t] = w;
-        }
-        uint4* d = reinterpret_cast<uint4*>(dst);
-        d[0] = make_uint4(o[0], o[1], o[2], o[3]);
-        d[1] = make_uint4(o[4], o[5], o[6], o[7]);
-    } else {
-        uint4* d = reinterpret_cast<uint4*>(dst);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) d[q] = make_uint4(cw[4 * q], cw[4 * q + 1], cw[4 * q + 2], cw[4 * q + 3]);
-    }
-}
-
-// Code j of an item of width B held in 2*B words.
-template <int B>
-__device__ __forceinline__ uint32_t item_code(const uint32_t* w, int j) {
-    if (B == 1) return (w[j >> 5] >> (j & 31)) & 1u;
-    if (B == 2) return ((w[j >> 5] >> (j & 31)) & 1u) | (((w[2 + (j >> 5)] >> (j & 31)) & 1u) << 1);
-    if (B == 4) return (w[j >> 3] >> (4 * (j & 7))) & 0xfu;
-    return (w[j >> 2] >> (8 * (j & 3))) & 0xffu;
-}
-
-// Load an item of width B (8-byte aligned for B = 1, 16-byte otherwise) into 2*B words.
-template <int B>
-__device__ __forceinline__ void load_item(const uint8_t* __restrict__ src, uint32_t* w) {
-    if (B == 1) {
-        uint2 v = *reinterpret_cast<const uint2*>(src);
-        w[0] = v.x; w[1] = v.y;
-    } else {
-#pragma unroll
-        for (int q = 0; q < B / 2; ++q) {
-            uint4 v = reinterpret_cast<const uint4*>(src)[q];
-            w[4 * q] = v.x; w[4 * q + 1] = v.y; w[4 * q + 2] = v.z; w[4 * q + 3] = v.w;
-        }
-    }
-}
-
-// Level L_b(u): 2u - 1 for b = 1, u - 2^(b-1) otherwise.
-template <int B>
-__device__ __forceinline__ int level_of(uint32_t u) {
-    return B == 1 ? (int)(2 * u) - 1 : (int)u - (1 << (B - 1));
-}
-
-// Column of item i of width w, given its column-end table cend (C entries,
-// nondecreasing) and a lower bound c0 on the answer.
-__device__ __forceinline__ int column_of(const uint16_t* cend, int cols, int c0, int i) {
-    int c = c0;
-    while (c < cols - 1 && (int)cend[c] <= i) ++c;
-    return c;
 }
 
 }  // namespace vbq

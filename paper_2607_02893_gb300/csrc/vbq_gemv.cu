@@ -126,11 +126,11 @@ struct __align__(16) TablesT : ActTab<NX> {
     int abort;                           // set by any role whose wait ran out
 };
 template <int NX> struct TablesCheck {
-    using T = TablesT<NX>;
-    static_assert(offsetof(T, full) % 8 == 0, "mbarriers are 8-byte aligned");
-    static_assert(offsetof(T, lut) == 0, "tables start at the aligned base");
-    static_assert(offsetof(T, x4z) % 16 == 0 && offsetof(T, xs) % 16 == 0 && offsetof(T, x4s) % 16 == 0 &&
-                  offsetof(T, slots) % 16 == 0, "16-byte table reads");
+    using A = ActTab<NX>;
+    static_assert(offsetof(A, lut) == 0, "tables start at the aligned base");
+    static_assert(offsetof(A, x4z) % 16 == 0 && offsetof(A, xs) % 16 == 0 && offsetof(A, x4s) % 16 == 0 &&
+                  sizeof(A) % 16 == 0, "16-byte table reads, and slots after the tables");
+    static_assert(SLOT_FLOATS * sizeof(float) % 16 == 0, "mbarriers, after the slots, are 8-byte aligned");
     static constexpr bool ok = true;
 };
 static_assert(TablesCheck<1>::ok && TablesCheck<2>::ok, "table layout");

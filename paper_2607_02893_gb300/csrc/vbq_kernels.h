@@ -8,18 +8,21 @@
 
 namespace vbq {
 
-// Pack-time kernels (vbq_pack.cu).
-cudaError_t launch_validate(const uint8_t* codes, const uint8_t* widths, int64_t N, int64_t K,
-                            uint32_t* err_flags, cudaStream_t s);
+// Pack-time kernels (vbq_pack.cu): per unit, item counts per width and warp
+// tasks (counts[5u ..]); then the blobs. *err (a word the host can read) is
+// set to 1 by launch_count for a width outside {1,2,4,8}, by launch_scatter
+// for a code >= 2^b of its group.
 cudaError_t launch_count(const uint8_t* widths, int64_t N, int G, int C, int nrb, int units,
-                         uint32_t* counts, cudaStream_t s);
+                         uint32_t* counts, uint32_t* err, cudaStream_t s);
 cudaError_t launch_scatter(const uint8_t* codes, const uint8_t* widths, const uint16_t* scales,
-                           const UnitHeader* headers, const LayoutView& L, uint8_t* blobs, cudaStream_t s);
+                           const uint32_t* counts, const LayoutView& L, uint8_t* blobs, uint32_t* err,
+                           cudaStream_t s);
 cudaError_t launch_dequant(const LayoutView& L, uint8_t* codes_out, uint8_t* widths_out,
                            uint16_t* scales_out, float* w_out, cudaStream_t s);
 
-// Quantisation (vbq_quant.cu): validation (bit 0 of err: a width outside
-// {1,2,4,8}; bit 1: a NaN weight), then codes and FP16 scales per group.
+// Quantisation (vbq_quant.cu): validation (err[0] set to 1 for a width outside
+// {1,2,4,8}, err[1] for a NaN weight; words the host can read), then codes and
+// FP16 scales per group.
 cudaError_t launch_quant_validate(const float* w, const uint8_t* widths, int64_t N, int64_t K, uint32_t* err,
                                   cudaStream_t s);
 cudaError_t launch_quantize(const float* w, const uint8_t* widths, int64_t N, int64_t K, uint8_t* codes,

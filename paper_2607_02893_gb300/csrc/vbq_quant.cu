@@ -171,7 +171,7 @@ __device__ __forceinline__ uint32_t one_bit_scale(float a0, float a1) {
     return near ? one_bit_scale_exact(a0, a1) : c;
 }
 
-// Width in {1, 2, 4, 8} for every group (bit 0) and no NaN weight (bit 1):
+// Width in {1, 2, 4, 8} for every group (else err[0] = 1) and no NaN weight (else err[1] = 1):
 // 16-byte loads over w and the widths as flat arrays.
 __global__ void quant_validate_kernel(const float* __restrict__ w, const uint8_t* __restrict__ widths,
                                       int64_t nweights, int64_t ngroups, uint32_t* err) {
@@ -191,7 +191,8 @@ __global__ void quant_validate_kernel(const float* __restrict__ w, const uint8_t
         const uint32_t b = widths[gi];
         if (b != 1 && b != 2 && b != 4 && b != 8) flags |= 1u;
     }
-    if (flags) atomicOr(err, flags);
+    if (flags & 1u) err[0] = 1u;
+    if (flags & 2u) err[1] = 1u;
 }
 
 __global__ void __launch_bounds__(QTHREADS) quantize_kernel(const float* __restrict__ w,
