@@ -21,16 +21,21 @@
 //   - the 1-bit mean: exact integer arithmetic when the fp64 tree is exact
 //     (see one_bit_scale), else the fp64 tree itself.
 //
-// One warp per group, two weights per lane (one 8-byte load; a warp reads the
-// group's 256 bytes in one coalesced request), several groups per warp in
-// flight.
+// A warp takes 16 groups at a time, four per 16-byte load and lane: eight
+// lanes hold a group, weights 4l .. 4l + 3 and 32 + 4l .. of it in lane l, so
+// loads and stores are whole 128- and 32-byte segments and a group's reduction
+// is three shuffles for four groups at once. The scale rounding (about 60
+// instructions) is done once per 16 groups, a group per lane, instead of once
+// per group by every lane.
 #include "vbq_kernels.h"
 
 namespace vbq {
 namespace {
 
 constexpr int QTHREADS = 256;            // 8 warps per block
-constexpr int QGROUPS = 8;               // groups in flight per warp
+constexpr int QLOADS = 4;                // loads of four groups in flight per warp
+constexpr int QGROUPS = 4 * QLOADS;      // groups per warp pass
+constexpr int64_t QKEEP_BYTES = 64 << 20;   // weights the validation leaves in L2 (129 MB) for the quantisation
 
 // FP16 bits of RN(S * 2^P) (S >= 0 an exact integer below 2^53), values
 // above 65504 saturating to 65504: integer round-half-even at the FP16
@@ -110,71 +115,108 @@ __device__ __noinline__ int code_magnitude_exact(float a, float sf, float hs, fl
     else if (a == lo) q -= q & 1;              // tie between k - 1 and k
     return min(q, qmax);
 }
-// The same with r an estimate of 1 / sf within 2^-22 relative: t = fl(a * r)
-// is within (a / sf) 2^-21 <= 2^-13 of the quotient (up to the 256 cap), so
-// when t is at least 0.0005 away from a half-integer, rint(t) is the answer;
-// otherwise (rarely) the exact thresholds decide.
-__device__ __forceinline__ int code_magnitude(float a, float sf, float hs, float r, int qmax) {
-    const float t = fminf(a * r, 256.f);
-    const float k = rintf(t);
-    if (fabsf(t - k) <= 0.4995f) return min((int)k, qmax);
-    return code_magnitude_exact(a, sf, hs, k, qmax);   // near a half-integer (rare)
-}
-
-// The 1-bit scale FP16(mean |w|) of a group held two weights per lane, with
-// the mean's sum taken as the balanced fp64 tree over neighbouring weights.
+// The 1-bit scale FP16(mean |w|) of a group in global memory, by the eight
+// lanes of mask (lane l of them: weights 4l .. and 32 + 4l ..), with the
+// mean's sum taken as the balanced fp64 tree over neighbouring weights.
 // When every nonzero |w| is a multiple of 2^L (L the smallest ulp exponent)
 // and the largest ulp exponent is at most L + 23, all partial sums of that
 // tree are multiples of 2^L below 2^(L + 53): the fp64 tree is exact, and the
 // exact integer sum S = sum |w| / 2^L (below 2^53) gives FP16(S * 2^(L - 6))
 // directly. Otherwise (a spread over 23 binades, or an infinity) the fp64
 // tree is evaluated as written.
-__device__ __noinline__ uint32_t one_bit_scale_exact(float a0, float a1) {
-    const uint32_t b0 = __float_as_uint(a0), b1 = __float_as_uint(a1);
-    const int e0 = (int)(b0 >> 23), e1 = (int)(b1 >> 23);           // biased exponents (a >= 0)
-    // ulp exponents of nonzero values (subnormals share the smallest normal's)
-    const int u0 = max(e0, 1) - 150, u1 = max(e1, 1) - 150;
-    const int lo = min(b0 ? u0 : 1000, b1 ? u1 : 1000), hi = max(b0 ? u0 : -1000, b1 ? u1 : -1000);
-    const int L = __reduce_min_sync(0xffffffffu, lo), H = __reduce_max_sync(0xffffffffu, hi);
-    const bool finite = __all_sync(0xffffffffu, e0 < 255 && e1 < 255);
+__device__ __noinline__ uint32_t one_bit_scale_exact(const float* group, int l, unsigned mask) {
+    const float4 f0 = reinterpret_cast<const float4*>(group)[l], f1 = reinterpret_cast<const float4*>(group)[8 + l];
+    const float a[8] = {fabsf(f0.x), fabsf(f0.y), fabsf(f0.z), fabsf(f0.w), fabsf(f1.x), fabsf(f1.y), fabsf(f1.z), fabsf(f1.w)};
+    int L = 1000, H = -1000;
+    bool finite = true;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const uint32_t b = __float_as_uint(a[i]);
+        const int e = (int)(b >> 23), u = max(e, 1) - 150;          // ulp exponent (subnormals share the smallest normal's)
+        if (b) { L = min(L, u); H = max(H, u); }
+        finite &= e < 255;
+    }
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+        L = min(L, __shfl_xor_sync(mask, L, o));
+        H = max(H, __shfl_xor_sync(mask, H, o));
+    }
+    finite = __all_sync(mask, finite);
     if (L == 1000) return 0u;                                        // all zero
     if (finite && H - L <= 23) {
-        const unsigned long long m0 = b0 ? (unsigned long long)((b0 & 0x7FFFFFu) | (e0 ? 0x800000u : 0u)) << (u0 - L) : 0ull;
-        const unsigned long long m1 = b1 ? (unsigned long long)((b1 & 0x7FFFFFu) | (e1 ? 0x800000u : 0u)) << (u1 - L) : 0ull;
-        unsigned long long S = m0 + m1;
+        unsigned long long S = 0;
 #pragma unroll
-        for (int off = 1; off < 32; off <<= 1) S += __shfl_xor_sync(0xffffffffu, S, off);
+        for (int i = 0; i < 8; ++i) {
+            const uint32_t b = __float_as_uint(a[i]);
+            const int e = (int)(b >> 23), u = max(e, 1) - 150;
+            if (b) S += (unsigned long long)((b & 0x7FFFFFu) | (e ? 0x800000u : 0u)) << (u - L);
+        }
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) S += __shfl_xor_sync(mask, S, o);
         return fp16_bits_of_scaled(S, L - 6);
     }
-    double p = (double)a0 + (double)a1;                              // leaves of the pairwise tree
+    // the pairwise tree: each half's 32 weights over its lanes, then the halves
+    double p = ((double)a[0] + (double)a[1]) + ((double)a[2] + (double)a[3]);
+    double q = ((double)a[4] + (double)a[5]) + ((double)a[6] + (double)a[7]);
 #pragma unroll
-    for (int off = 1; off < 32; off <<= 1) p += __shfl_xor_sync(0xffffffffu, p, off);
-    return fp16_bits_sat(p * (1.0 / GROUP));                         // exact division by 64
+    for (int o = 1; o < 8; o <<= 1) {
+        p += __shfl_xor_sync(mask, p, o);
+        q += __shfl_xor_sync(mask, q, o);
+    }
+    return fp16_bits_sat((p + q) * (1.0 / GROUP));                   // exact division by 64
 }
 
-// The same scale, first from an fp32 tree of the same shape: its sum is
-// within 6 * 2^-24 (depth times unit roundoff) of the exact sum of the
-// non-negative |w|, so its FP16 rounding is the exact mean's unless an FP16
-// midpoint lies within 2^-20 of the fp32 mean; only then (rarely) the exact
-// evaluation runs. Warp-uniform: every lane holds the same fp32 sum.
-__device__ __forceinline__ uint32_t one_bit_scale(float a0, float a1) {
-    float t = a0 + a1;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+// The same scale from t, an fp32 tree of depth 6 over the group's |w|: within
+// 6 * 2^-24 (depth times unit roundoff) of the exact sum of the non-negative
+// values, so its FP16 rounding is the exact mean's unless an FP16 midpoint
+// lies within 2^-20 of the fp32 mean; then (rarely) near is set and the exact
+// evaluation has to run.
+__device__ __forceinline__ uint32_t one_bit_scale(float t, bool& near) {
+    near = false;
     if (isinf(t)) return 0x7BFFu;                      // the exact mean is far above 65504 too
     const float mean = t * (1.f / GROUP);              // exact
-    uint32_t c = min((uint32_t)__half_as_ushort(__float2half_rn(mean)), 0x7BFFu);
+    const uint32_t c = min((uint32_t)__half_as_ushort(__float2half_rn(mean)), 0x7BFFu);
     const float cv = __half2float(__ushort_as_half((uint16_t)c)), err = mean * 0x1p-20f;
-    bool near = false;
     if (c < 0x7BFFu) near |= fabsf(mean - 0.5f * (cv + __half2float(__ushort_as_half((uint16_t)(c + 1))))) <= err;
     if (c > 0u) near |= fabsf(mean - 0.5f * (cv + __half2float(__ushort_as_half((uint16_t)(c - 1))))) <= err;
-    return near ? one_bit_scale_exact(a0, a1) : c;
+    return c;
 }
 
-// Width in {1, 2, 4, 8} for every group (else err[0] = 1) and no NaN weight (else err[1] = 1):
-// 16-byte loads over w and the widths as flat arrays.
+// Codes of four weights as bytes (b >= 2), from r, an estimate of 1 / sf within
+// 2^-22 relative (0 for sf = 0: every code is z). t = fl(v r), clipped to
+// +-qmax, is within 2^-13 of the clipped quotient, and adding 1.5 * 2^23 + z
+// rounds it half to even to the integer q and leaves q + z in the low byte.
+// That is the answer whenever t is at least 0.0005 from a half-integer;
+// otherwise (rarely) the exact thresholds decide.
+__device__ __forceinline__ uint32_t codes4(float4 v, float r, float sf, float qmaxf, float magic) {
+    const float x[4] = {v.x, v.y, v.z, v.w};
+    uint32_t u[4];
+    float worst = 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float t = fminf(fmaxf(__fmul_rn(x[i], r), -qmaxf), qmaxf);
+        const float m = __fadd_rn(t, magic);
+        worst = fmaxf(worst, fabsf(__fsub_rn(t, __fsub_rn(m, magic))));
+        u[i] = __float_as_uint(m);
+    }
+    if (worst > 0.4995f && r != 0.f) {                 // some weight near a half-integer
+        const int z = (int)(magic - 12582912.f);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float a = fabsf(x[i]);
+            const int q = code_magnitude_exact(a, sf, 0.5f * sf, rintf(fminf(a * r, 256.f)), (int)qmaxf);
+            u[i] = (uint32_t)(z + (x[i] < 0.f ? -q : q));
+        }
+    }
+    return __byte_perm(__byte_perm(u[0], u[1], 0x0040), __byte_perm(u[2], u[3], 0x0040), 0x5410);
+}
+
+// Width in {1, 2, 4, 8} for every group (else err[0] = 1) and no NaN weight
+// (else err[1] = 1): 16-byte loads over w and the widths as flat arrays. The
+// weights from `keep` on are loaded to stay in L2: quantize_kernel, which
+// walks the groups from the last, finds them there.
 __global__ void quant_validate_kernel(const float* __restrict__ w, const uint8_t* __restrict__ widths,
-                                      int64_t nweights, int64_t ngroups, uint32_t* err) {
+                                      int64_t nweights, int64_t ngroups, int64_t keep, uint32_t* err) {
     uint32_t flags = 0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x, t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t n4 = nweights / 4;                    // K % 64 == 0, so a whole number of float4
@@ -182,7 +224,10 @@ __global__ void quant_validate_kernel(const float* __restrict__ w, const uint8_t
     for (int64_t i = t0; i < n4; i += 4 * stride) {
         float4 v[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) v[j] = i + j * stride < n4 ? __ldcs(w4 + i + j * stride) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int j = 0; j < 4; ++j) {
+            const int64_t k = i + j * stride;
+            v[j] = k >= n4 ? make_float4(0.f, 0.f, 0.f, 0.f) : 4 * k < keep ? __ldcs(w4 + k) : __ldg(w4 + k);
+        }
 #pragma unroll
         for (int j = 0; j < 4; ++j)
             if (isnan(v[j].x) || isnan(v[j].y) || isnan(v[j].z) || isnan(v[j].w)) flags |= 2u;
@@ -195,59 +240,89 @@ __global__ void quant_validate_kernel(const float* __restrict__ w, const uint8_t
     if (flags & 2u) err[1] = 1u;
 }
 
-__global__ void __launch_bounds__(QTHREADS) quantize_kernel(const float* __restrict__ w,
+// 14336 x 4096 main: 101 -> 56 us (with the validation pass 146 -> 94).
+__global__ void __launch_bounds__(QTHREADS, 3) quantize_kernel(const float* __restrict__ w,
                                                             const uint8_t* __restrict__ widths, int64_t ngroups,
                                                             uint8_t* __restrict__ codes, uint16_t* __restrict__ scales) {
-    const int lane = threadIdx.x & 31;
+    constexpr unsigned ALL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, l = lane & 7, sub = lane >> 3;      // lane l of the load's group `sub`
     const int64_t warps = (int64_t)gridDim.x * (QTHREADS >> 5);
-    for (int64_t g0 = ((int64_t)blockIdx.x * (QTHREADS >> 5) + (threadIdx.x >> 5)) * QGROUPS; g0 < ngroups;
-         g0 += warps * QGROUPS) {
-        float2 v[QGROUPS];
-        uint32_t bw[QGROUPS];
+    const int64_t chunks = (ngroups + QGROUPS - 1) / QGROUPS;
+    for (int64_t ck = (int64_t)blockIdx.x * (QTHREADS >> 5) + (threadIdx.x >> 5); ck < chunks; ck += warps) {
+        const int64_t g0 = (chunks - 1 - ck) * QGROUPS;                    // from the last (see quant_validate_kernel)
+        const int ng = (int)min((int64_t)QGROUPS, ngroups - g0);
+        // lane j < 16 owns group g0 + j's scale
+        const uint32_t bw = lane < ng ? widths[g0 + lane] : 2u;
+        float4 v[QLOADS][2];
 #pragma unroll
-        for (int j = 0; j < QGROUPS; ++j) {     // loads first: QGROUPS groups in flight
-            const int64_t gi = g0 + j < ngroups ? g0 + j : g0;
-            v[j] = __ldcs(reinterpret_cast<const float2*>(w + gi * GROUP) + lane);
-            bw[j] = widths[gi];
+        for (int k = 0; k < QLOADS; ++k) {
+            const int64_t gi = g0 + min(4 * k + sub, ng - 1);
+            const float4* src = reinterpret_cast<const float4*>(w + gi * GROUP);
+            v[k][0] = __ldcs(src + l);
+            v[k][1] = __ldcs(src + 8 + l);
         }
+        // max|w| and the fp32 tree of |w| of group 4k + sub; lane (4k + sub) keeps its own group's
+        float gmax = 0.f, gsum = 0.f;
 #pragma unroll
-        for (int j = 0; j < QGROUPS; ++j) {
-            const int64_t gi = g0 + j;
-            if (gi >= ngroups) break;           // warp-uniform
-            const float a0 = fabsf(v[j].x), a1 = fabsf(v[j].y);
-            uint32_t sbits, u0, u1;
-            if (bw[j] == 1) {
-                sbits = one_bit_scale(a0, a1);
-                u0 = v[j].x >= 0.f;
-                u1 = v[j].y >= 0.f;
-            } else {
-                const int qmax = (1 << (bw[j] - 1)) - 1, z = 1 << (bw[j] - 1);
-                float m = fmaxf(a0, a1);
+        for (int k = 0; k < QLOADS; ++k) {
+            const float4 p = v[k][0], q = v[k][1];
+            float m = fmaxf(fmaxf(fmaxf(fabsf(p.x), fabsf(p.y)), fmaxf(fabsf(p.z), fabsf(p.w))),
+                            fmaxf(fmaxf(fabsf(q.x), fabsf(q.y)), fmaxf(fabsf(q.z), fabsf(q.w))));
+            float t = ((fabsf(p.x) + fabsf(p.y)) + (fabsf(p.z) + fabsf(p.w))) +
+                      ((fabsf(q.x) + fabsf(q.y)) + (fabsf(q.z) + fabsf(q.w)));
 #pragma unroll
-                for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-                sbits = fp16_bits_of_quotient(m, qmax);
-                const float sf = __half2float(__ushort_as_half((uint16_t)sbits));
-                if (sf == 0.f) {
-                    u0 = u1 = (uint32_t)z;
-                } else {
-                    const float r = rcp_estimate(sf), hs = 0.5f * sf;
-                    const int q0 = code_magnitude(a0, sf, hs, r, qmax), q1 = code_magnitude(a1, sf, hs, r, qmax);
-                    u0 = (uint32_t)(z + (v[j].x < 0.f ? -q0 : q0));
-                    u1 = (uint32_t)(z + (v[j].y < 0.f ? -q1 : q1));
-                }
+            for (int o = 1; o < 8; o <<= 1) {
+                m = fmaxf(m, __shfl_xor_sync(ALL, m, o));
+                t += __shfl_xor_sync(ALL, t, o);
             }
-            reinterpret_cast<uint16_t*>(codes + gi * GROUP)[lane] = (uint16_t)(u0 | (u1 << 8));
-            if (lane == 0) scales[gi] = (uint16_t)sbits;
+            const float mk = __shfl_sync(ALL, m, 8 * (lane & 3)), tk = __shfl_sync(ALL, t, 8 * (lane & 3));
+            if ((lane >> 2) == k) { gmax = mk; gsum = tk; }
+        }
+        bool near = false;
+        const int qmax = (1 << (bw - 1)) - 1;
+        uint32_t sbits = bw == 1 ? one_bit_scale(gsum, near) : fp16_bits_of_quotient(gmax, qmax);
+        // groups whose 1-bit mean is near an FP16 midpoint: exactly, by their eight lanes
+        for (uint32_t todo = __ballot_sync(ALL, near && lane < ng); todo; todo &= todo - 1) {
+            const int j = __ffs(todo) - 1;
+            uint32_t ex = 0;
+            if (lane < 8) ex = one_bit_scale_exact(w + (g0 + j) * GROUP, lane, 0xFFu);
+            ex = __shfl_sync(ALL, ex, 0);
+            if (lane == j) sbits = ex;
+        }
+        if (lane < ng) scales[g0 + lane] = (uint16_t)sbits;
+        const float sf = __half2float(__ushort_as_half((uint16_t)sbits));
+        const float r = sf == 0.f ? 0.f : rcp_estimate(sf);
+#pragma unroll
+        for (int k = 0; k < QLOADS; ++k) {
+            const int j = 4 * k + sub;
+            const uint32_t bj = __shfl_sync(ALL, bw, j);
+            const float sj = __shfl_sync(ALL, sf, j), rj = __shfl_sync(ALL, r, j);
+            uint32_t lo, hi;
+            if (bj == 1) {
+                const float4 p = v[k][0], q = v[k][1];
+                lo = (p.x >= 0.f ? 1u : 0u) | (p.y >= 0.f ? 0x100u : 0u) | (p.z >= 0.f ? 0x10000u : 0u) | (p.w >= 0.f ? 0x1000000u : 0u);
+                hi = (q.x >= 0.f ? 1u : 0u) | (q.y >= 0.f ? 0x100u : 0u) | (q.z >= 0.f ? 0x10000u : 0u) | (q.w >= 0.f ? 0x1000000u : 0u);
+            } else {
+                const int z = 1 << (bj - 1);
+                const float qm = (float)(z - 1), magic = 12582912.f + (float)z;
+                lo = codes4(v[k][0], rj, sj, qm, magic);
+                hi = codes4(v[k][1], rj, sj, qm, magic);
+            }
+            if (j < ng) {
+                uint32_t* dst = reinterpret_cast<uint32_t*>(codes + (g0 + j) * GROUP);
+                dst[l] = lo;
+                dst[8 + l] = hi;
+            }
         }
     }
 }
 
-int grid_for(int64_t ngroups, int warps_per_block, int per_warp) {
+int grid_for(int64_t ngroups, int warps_per_block, int per_warp, int blocks_per_sm) {
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t need = (ngroups + (int64_t)warps_per_block * per_warp - 1) / ((int64_t)warps_per_block * per_warp);
-    const int64_t cap = (int64_t)sms * 8;       // 8 blocks of 8 warps per SM
+    const int64_t cap = (int64_t)sms * blocks_per_sm;       // one resident wave, grid-stride
     return (int)(need < cap ? (need > 0 ? need : 1) : cap);
 }
 
@@ -256,14 +331,15 @@ int grid_for(int64_t ngroups, int warps_per_block, int per_warp) {
 cudaError_t launch_quant_validate(const float* w, const uint8_t* widths, int64_t N, int64_t K, uint32_t* err,
                                   cudaStream_t s) {
     const int64_t ngroups = N * (K / GROUP);
-    quant_validate_kernel<<<grid_for(N * K / 4, QTHREADS, 4), QTHREADS, 0, s>>>(w, widths, N * K, ngroups, err);
+    const int64_t keep = N * K - QKEEP_BYTES / 4;
+    quant_validate_kernel<<<grid_for(N * K / 4, QTHREADS, 4, 4), QTHREADS, 0, s>>>(w, widths, N * K, ngroups, keep, err);
     return cudaGetLastError();
 }
 
 cudaError_t launch_quantize(const float* w, const uint8_t* widths, int64_t N, int64_t K, uint8_t* codes,
                             uint16_t* scales, cudaStream_t s) {
     const int64_t ngroups = N * (K / GROUP);
-    quantize_kernel<<<grid_for(ngroups, QTHREADS / 32, QGROUPS), QTHREADS, 0, s>>>(w, widths, ngroups, codes, scales);
+    quantize_kernel<<<grid_for(ngroups, QTHREADS / 32, QGROUPS, 3), QTHREADS, 0, s>>>(w, widths, ngroups, codes, scales);
     return cudaGetLastError();
 }
 
