@@ -206,11 +206,9 @@ vbq_status_t vbq_gemv(const vbq_layout* layout, const uint16_t* x, float* y,
  * batch-1 table kernel, two rows per launch (both rows share every lookup
  * address and decoded code) and a single row for an odd count, each row
  * computed as vbq_gemv computes it; or the tensor cores (chosen for layouts
- * heavy in 4- and 8-bit groups). For B >= 5 the product runs on the tensor
- * cores:
- * activations are scaled per (row, group column) by a power of two into fp16
- * range (values below 2^-14 of that scale lose low bits), weights enter as
- * exact levels, products and fp32 accumulation as in vbq_gemv. Y needs no
+ * heavy in 4- and 8-bit groups, and for most mixes from three
+ * rows on). For B >= 5 the product runs on the tensor cores: activations as
+ * they are (BF16), weights as exact levels, fp32 accumulation. Y needs no
  * zeroing; the same split-K workspace and ordering rules as vbq_gemv apply
  * (calls sharing a layout must not overlap on the GPU), and the kernels are
  * launched the same way.

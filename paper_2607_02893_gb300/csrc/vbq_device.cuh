@@ -119,10 +119,7 @@ __device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
 
 __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
 
-// y += v on a shared-memory float (32-bit shared address) / a global float.
-__device__ __forceinline__ void red_shared(uint32_t addr, float v) {
-    asm volatile("red.shared.add.f32 [%0], %1;" :: "r"(addr), "f"(v) : "memory");
-}
+// y += v on a global float.
 __device__ __forceinline__ void red_global(float* p, float v) {
     asm volatile("red.global.add.f32 [%0], %1;" :: "l"(p), "f"(v) : "memory");
 }
@@ -265,8 +262,9 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_
 __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, uint32_t abort_addr, uint32_t nap_ns = 0) {
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_addr, nap_ns));
 }
-// Plain bounded wait (no abort flag), for the copier's final drain.
+// Plain bounded wait (no abort flag), for the copiers' final drain.
 __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity) {
+    if (mbar_try_wait(bar, parity)) return true;
     const unsigned long long t0 = global_ns();
     while (!mbar_try_wait_sleep(bar, parity)) {
         if (global_ns() - t0 > WAIT_LIMIT_NS) return false;

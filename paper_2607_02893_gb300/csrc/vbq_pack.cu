@@ -128,8 +128,8 @@ __global__ void __launch_bounds__(RB) count_kernel(const uint8_t* __restrict__ w
 // position (bin b holds positions b, b + 16, ...; the first nt % 16 bins one
 // more than the rest, so the positions are exactly 0 .. nt - 1; bins b and
 // b + 8 together are a warp's share when tw = 8). The costs are the batch-1
-// kernel's measured time per group and width (COST_ONE in vbq_plan.cu: 5.33,
-// 7.02, 9.98, 14.0 units for 1, 2, 4, 8 bits) times a task's items: a task
+// kernel's time per group and width (measured: 5.33, 7.02, 9.98, 14.0 units for
+// 1, 2, 4, 8 bits) times a task's items: a task
 // costs its full span even when shorter, since idle lanes repeat its first
 // item. The order does not change any result: every group has its own slot.
 // One warp: lane b < 16 is bin b, and the least-loaded bin is one warp
