@@ -202,11 +202,17 @@ vbq_status_t vbq_pack(const uint8_t* codes, const uint8_t* bitwidths, const uint
         d_scales = static_cast<uint16_t*>(ps);
     }
 
-    // 1. plan: row blocks x slabs (the counting kernel also checks the widths). Take the widest slab (C in 16..1) that gives
-    // at least half as many units as SMs and whose largest unit blob fits a
-    // stage. (Wider units cost less per group than the imbalance they leave:
-    // measured on 1B- and 9B-class shapes, 4096^2 takes 5.8 us with C = 16
-    // against 6.6 us with C = 4, the width a 3-units-per-SM rule picks.)
+    // 1. plan: row blocks x slabs of C columns (the counting kernel also checks
+    // the widths). First the narrowest slab (2, 4 or 8 columns) with which the
+    // batch-1 product runs one unit per block, all at once, a row block's slabs a
+    // cluster of at most 8 (else 16) blocks (vbq::unit_plan_fits): measured at
+    // batch 1 / 4 / 16 against the rule below (us in a graph), 5632x2048 4.2 /
+    // 7.2 / 9.3 with C = 16, 3.7 / 5.6 / 7.7 with C = 8; 1024x4096 (C = 4) 3.0 /
+    // 4.1 / 5.8, (C = 8) 3.0 / 4.0 / 5.2; 256x2048 (C = 1) 2.9, (C = 4) 2.2 at
+    // batch 1. Larger matrices take the widest slab (C in 16..1) that gives at
+    // least half as many units as SMs (wider units cost less per group than the
+    // imbalance they leave: 6144x4096 5.6 / 8.1 / 11.5 with C = 16, 5.2 / 9.3 /
+    // 14.1 with C = 8). Either way a unit's blob has to fit a stage.
     int dev = 0, sms = 0;
     VBQ_CUDA(cudaGetDevice(&dev));
     VBQ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -216,11 +222,25 @@ vbq_status_t vbq_pack(const uint8_t* codes, const uint8_t* bitwidths, const uint
     int C = 0;
     int64_t S = 0, units = 0;
     uint32_t max16 = 0;
-    for (int cand : {16, 8, 4, 2, 1}) {
-        if (cand > vbq::MAX_C || (cand > G && cand != 1)) continue;
+    std::vector<int> cands;
+    for (int most : {8, vbq::MAX_CLUSTER}) {
+        for (int c : {2, 4, 8}) {
+            const int64_t Sc = (G + c - 1) / c;
+            if (c <= G && cands.empty() && Sc <= most && vbq::unit_plan_fits(c, Sc, nrb * Sc, (int64_t)ngroups, sms)) cands.push_back(c);
+        }
+    }
+    bool widest = true;
+    for (int c : {16, 8, 4, 2, 1}) {
+        if ((c > G || 2 * nrb * ((G + c - 1) / c) < sms) && c != 1) continue;    // fewer units than half the SMs: narrower slabs
+        // where the unit kernel will not run (see unit_neighbours), its plan only
+        // where that is the narrower one
+        if (widest && !cands.empty() && c < cands[0] && !vbq::unit_neighbours(G)) cands.clear();
+        widest = false;
+        if (cands.empty() || cands[0] != c) cands.push_back(c);
+    }
+    for (const int cand : cands) {
         const int64_t Sc = (G + cand - 1) / cand, uc = nrb * Sc;
-        const bool last = (cand == 1);
-        if (!last && 2 * uc < sms) continue;          // fewer units than half the SMs: narrower slabs
+        const bool last = cand == cands.back();
         if (uc > (1LL << 31) - 2) return fail(VBQ_ERR_UNSUPPORTED, "too many units");
         void* dc = nullptr;
         std::vector<uint32_t> cnt((size_t)uc * 5);

@@ -1343,23 +1343,11 @@ __global__ void __launch_bounds__(CH_THREADS, 1) gemv_chain_kernel(const ChainIt
 // mbarrier there), which adds them in slab order and stores y once: no
 // zeroing, flags, atomics or control words, and the same bits on every call.
 // Per product, in a graph of dependent products (us, persistent kernel before
-// -> this): 768x768 3.04 -> 2.32, 2048x768 3.71 -> 2.31, 768x2048 3.33 -> 2.45;
-// the 85 products of the ~131M decode step 265 -> 208 us.
+// -> this, with the slabs planned for it): 768x768 3.04 -> 2.22, 2048x768 3.71
+// -> 2.34, 2048x2048 3.83 -> 2.83, 256x2048 2.86 -> 2.24, 5632x2048 4.12 -> 3.72; the 85
+// products of the ~131M decode step 265 -> 203 us.
 // ---------------------------------------------------------------------------
 constexpr int U1_THREADS = NCT;          // every warp consumes
-constexpr int MAX_CLUSTER = 16;          // blocks of one row block: its slabs (over 8 is opt-in)
-
-// Layouts for the unit kernel: units of at most 2 columns (wider units come
-// from larger matrices, where a cluster launched between persistent blocks
-// gains nothing: a ~9B layer whose 1024x4096 products, 4-column units in
-// clusters of 16, ran here took 45.4 against 45.1 us), a row block's slabs
-// within the largest cluster, and every cluster resident at once (two blocks
-// per SM, less what clusters leave unused of a GPC's SMs: 276..296 blocks fit
-// for up to 8 slabs, 196..253 above; as several waves of clusters 14336x4096
-// takes 8.3 -> 10.9 us).
-inline bool unit_per_block(const LayoutView& L, int sms) {
-    return L.C <= 2 && L.S <= MAX_CLUSTER && 4 * L.units <= (L.S <= 8 ? 7 : 5) * sms;
-}
 
 struct __align__(16) TablesU : ActTab<1> {
     float slots[SLOT_FLOATS];
@@ -1512,7 +1500,7 @@ cudaError_t launch_gemv1(const LayoutView& L, const uint16_t* x, float* y, cudaS
     cudaError_t e = prep.get(gemv1_kernel<NX, MODE, SW>, gemv1_smem<NX>(), &sms);
     if (e != cudaSuccess) return e;
     if constexpr (NX == 1) {
-        if (unit_per_block(L, sms)) return launch_gemv1_unit<MODE, SW>(L, x, y, s, dep, h, gu);
+        if (runs_unit_per_block(L, sms)) return launch_gemv1_unit<MODE, SW>(L, x, y, s, dep, h, gu);
     }
     const int grid = L.units < sms ? L.units : sms;
     cudaLaunchConfig_t cfg = {};

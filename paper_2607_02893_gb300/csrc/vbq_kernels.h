@@ -40,6 +40,33 @@ cudaError_t launch_soft_quant(const float* w, const float* logits, const float* 
 constexpr int GEMV1_MAX_B = 4;
 bool tables_for_batch(const LayoutView& L, int B);
 
+// Layouts planned so that the batch-1 product can run one unit per block, a row
+// block's S slabs a cluster (gemv1_unit_kernel, vbq_gemv.cu): units of at most
+// 8 columns (a wider unit's 2048 groups on one block's 16 warps take longer
+// than the hand-over saves: 4096x4096 as 128 16-column units 4.6 -> 5.1 us),
+// clusters of at most 16 blocks, every cluster resident at once (two blocks
+// per SM, less what clusters leave unused of a GPC's SMs: 276..296 blocks fit
+// for up to 8 slabs, 196..253 above; in several waves of clusters 14336x4096
+// takes 8.3 -> 10.9 us), and fewer than 200,000 groups (below).
+constexpr int MAX_CLUSTER = 16;
+constexpr int64_t UNIT_MAX_GROUPS = 200000;
+inline bool unit_plan_fits(int64_t C, int64_t S, int64_t units, int64_t groups, int sms) {
+    return C <= 8 && S <= MAX_CLUSTER && groups < UNIT_MAX_GROUPS && 4 * units <= (S <= 8 ? 7 : 5) * (int64_t)sms;
+}
+// Whether it does run them so. The unit kernel gains where its neighbours on
+// the stream are unit kernels too, whose blocks share SMs with it; next to a
+// persistent block of 226 KB its clusters wait for whole SMs. A ~9B layer's
+// fused products (4096x4096, 262,144 groups, between 6144x4096 and
+// 28672x4096) take 36.9 us with 4096x4096 on the persistent kernel and 39.0 on
+// this one, and its 1024x4096 products among 4096x4096 ones cost the unfused
+// layer 0.5 us; a ~1B layer, all but the head below the line, takes 22.8
+// instead of 26.1. So a matrix stays off it when it, or a square matrix on its
+// input (what its neighbours are like), has 200,000 groups or more.
+inline bool unit_neighbours(int64_t G) { return GROUP * G * G < UNIT_MAX_GROUPS; }
+inline bool runs_unit_per_block(const LayoutView& L, int sms) {
+    return unit_neighbours(L.G) && unit_plan_fits(L.C, L.S, L.units, L.N * L.G, sms);
+}
+
 // Products (vbq_gemv.cu). Y is B x N, overwritten (no zeroing needed).
 cudaError_t launch_gemv(const LayoutView& L, const uint16_t* X, float* Y, int B, cudaStream_t s);
 
