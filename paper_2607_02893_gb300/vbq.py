@@ -94,11 +94,27 @@ def _ptr(t) -> Optional[int]:
     return t.data_ptr()
 
 
+_current_raw_stream = None
+
+
+def _raw_stream_getter():
+    """Returns a function giving torch's current stream of the current device as an integer handle."""
+    import torch
+    get, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+    if get is None or device is None:
+        return lambda: torch.cuda.current_stream().cuda_stream
+    # the handle without a Stream object around it, which took 2.8 us of a 7.6 us vbq_gemv call
+    return lambda: get(device())
+
+
 def _stream(stream, *tensors) -> Optional[int]:
     if stream is None:
-        import torch
-        if any(getattr(t, "is_cuda", False) for t in tensors if t is not None):
-            return torch.cuda.current_stream().cuda_stream or None
+        global _current_raw_stream
+        for t in tensors:
+            if getattr(t, "is_cuda", False):
+                if _current_raw_stream is None:
+                    _current_raw_stream = _raw_stream_getter()
+                return _current_raw_stream() or None
         return None
     if isinstance(stream, int):
         return stream or None
@@ -128,7 +144,7 @@ class Layout:
     def _as_parameter_(self):
         if not self.handle:
             raise ValueError("layout already freed")
-        return ctypes.c_void_p(self.handle)
+        return self.handle
 
 
 def vbq_quantize(w, bitwidths, codes_out=None, scales_out=None, stream=None):
