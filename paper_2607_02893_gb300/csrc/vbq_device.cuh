@@ -275,6 +275,38 @@ __device__ __forceinline__ void raise_abort(int* abort_flag) {
     atomicOr(&g_device_status, VBQ_DEVICE_TIMEOUT);
     *reinterpret_cast<volatile int*>(abort_flag) = 1;
 }
+// Thread-block clusters: another block's shared memory.
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+// Bounded wait for other blocks' st.async on this block's barrier. Longer than
+// any of their own waits: every block of the cluster sends its sums even when
+// a wait of its own ran out, so the receiver never exits before they land.
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity) {
+    const unsigned long long t0 = global_ns();
+    for (;;) {
+        uint32_t ok;
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
+                     "selp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(ok) : "r"(bar), "r"(parity), "n"(SUSPEND_HINT_NS) : "memory");
+        if (ok) return true;
+        if (global_ns() - t0 > 4 * WAIT_LIMIT_NS) return false;
+    }
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// One float into another block's shared memory, counted (4 bytes) on that block's barrier.
+__device__ __forceinline__ void st_async_f32(uint32_t dst, float v, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
+                 :: "r"(dst), "r"(__float_as_uint(v)), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void st_async_f32x4(uint32_t dst, float4 v, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+                 :: "r"(dst), "r"(__float_as_uint(v.x)), "r"(__float_as_uint(v.y)), "r"(__float_as_uint(v.z)),
+                    "r"(__float_as_uint(v.w)), "r"(bar) : "memory");
+}
 // One thread: expect `bytes` on the barrier and start the bulk copy.
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(bar), "r"(bytes) : "memory");
@@ -285,25 +317,6 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
 __device__ __forceinline__ void issue_unit(const LayoutView& L, int u, uint32_t dst, uint32_t bar) {
     const uint32_t o0 = L.blob_off[u], o1 = L.blob_off[u + 1];
     bulk_load(dst, L.blobs + (int64_t)o0 * 16, (o1 - o0) * 16, bar);
-}
-
-// Split-K: true once every row block this block adds a slab s > 0 into has
-// been zeroed in this call (flag == epoch), within the wait limit. A whole warp:
-// lane i watches units u_begin + i, + 32, ..., so one round trip covers them
-// all; the flags are read with acquire loads.
-__device__ __forceinline__ bool split_k_flags_ready(const LayoutView& L, uint32_t epoch, int u_begin, int u_end,
-                                                    int lane) {
-    bool seen = true;
-    const unsigned long long t0 = global_ns();
-    for (int u = u_begin + lane; u < u_end && seen; u += 32) {
-        if (u >= L.nrb) {               // slab > 0
-            const uint32_t* f = L.ctl + 2 + (u % L.nrb);
-            while (!(seen = ld_acquire_gpu(f) == epoch))
-                if (global_ns() - t0 > WAIT_LIMIT_NS) break;
-        }
-    }
-    __syncwarp();                       // every lane's later additions after every acquire
-    return __all_sync(0xffffffffu, seen);
 }
 
 }  // namespace

@@ -62,6 +62,7 @@ struct __align__(16) TablesB {
     float acc[NCWB][NB / 8][RB][8];             // per warp: the unit's row sums, 8 batch rows together
     unsigned long long full;                    // blob landed
     unsigned long long empty;                   // every consumer warp is done with the blob
+    unsigned long long sums;                    // clusters: the other slabs' sums of this block's rows landed
     uint32_t consts[12];                        // DecodeConsts
     int abort;
     uint32_t sk_ok;                             // the control warp's split-K flag check, passed on
@@ -89,6 +90,9 @@ __device__ __forceinline__ void mma16816_z(float (&d)[4], const uint32_t (&a)[4]
 
 __device__ __forceinline__ void sts_f32x2(uint32_t addr, float2 v) {
     asm volatile("st.shared.v2.f32 [%0], {%1, %2};" :: "r"(addr), "f"(v.x), "f"(v.y) : "memory");
+}
+__device__ __forceinline__ void sts_f32x4(uint32_t addr, float4 v) {
+    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" :: "r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
 }
 __device__ __forceinline__ float2 lds_f32x2_ordered(uint32_t addr) {
     float2 v;
@@ -273,17 +277,17 @@ __device__ __forceinline__ Deal deal_columns(int cols, int cw) {
     return Deal{cw >> lg, NCWB >> lg, 1 << lg, cw & ((1 << lg) - 1)};
 }
 
-// One warp's share of a unit (blob at sblob, activations of its slab at x);
-// xb holds the first column's activations.
+// One warp's share of columns [c_lo, c_lo + cols) of a unit (blob at sblob,
+// activations of its slab at x); xb holds the first column's activations.
 template <int NB>
-__device__ __forceinline__ void consume_unit_b(const DecodeConsts& K, uint32_t sblob, int C, int cols, const Deal& dl,
+__device__ __forceinline__ void consume_unit_b(const DecodeConsts& K, uint32_t sblob, int C, int c_lo, int cols, const Deal& dl,
                                                uint32_t (&xb)[NB], const uint16_t* __restrict__ x, int64_t Kx, int B,
                                                uint32_t acc, int lane) {
     const int g = lane >> 2, t = lane & 3, sh = 8 * (t & 1);
     const uint4 h0 = lds_u32x4(sblob), h1 = lds_u32x4(sblob + 16), h2 = lds_u32x4(sblob + 32);
     const uint32_t cc = sblob + (h2.x & 0xFFFF) * 16;
     const uint32_t my = acc + 8u * t;
-    for (int c = dl.c0; c < cols; c += dl.step) {
+    for (int c = c_lo + dl.c0; c < c_lo + cols; c += dl.step) {
         int s[4], e[4];
 #pragma unroll
         for (int w = 0; w < 4; ++w) {
@@ -306,7 +310,7 @@ __device__ __forceinline__ void consume_unit_b(const DecodeConsts& K, uint32_t s
             done += (n + 15) >> 4;
         }
         __syncwarp();                    // the next column's additions follow this one's (other lanes hold its rows)
-        if (c + dl.step < cols) load_acts<NB>(xb, x + (int64_t)(c + dl.step) * GROUP, Kx, B, g, t);
+        if (c + dl.step < c_lo + cols) load_acts<NB>(xb, x + (int64_t)(c + dl.step) * GROUP, Kx, B, g, t);
     }
 }
 
@@ -344,29 +348,118 @@ __device__ __forceinline__ void flush_rows(TablesB<NB>& T, const LayoutView& L, 
     }
 }
 
+// The slabs of a row block as one cluster (CL): block `rank` holds slab rank's
+// unit, and owns rows [rank * own, (rank + 1) * own) of the row block. Once
+// every block of the cluster is done with its blob (the cluster barrier before
+// this), each sends its sums of the others' rows into their stages (st.async,
+// counted on their `sums` barriers), adds the S sums of its own rows in slab
+// order and stores them: no zeroing, flags or global additions, and the same
+// bits on every call. Slab k's sums of a block's row i sit at ((k * own + i) *
+// NB) floats. write is false after a wait that ran out.
+__host__ __device__ inline int cluster_rows(int S) { return (RB + S - 1) / S; }
 template <int NB>
+__device__ __forceinline__ void flush_cluster(TablesB<NB>& T, uint32_t stage, const LayoutView& L, float* __restrict__ Y, int B,
+                                              int rb, int rank, int ct, bool write) {
+    const int rows = min(RB, (int)(L.N - (int64_t)rb * RB)), own = cluster_rows(L.S);
+    const uint32_t sums = smem_u32(&T.sums);
+    const int r = ct >> 1, q = ct & 1, to = r / own, i = r - to * own;
+#pragma unroll
+    for (int n = 0; n < NB / 8; ++n) {
+        const uint32_t at = smem_u32(&T.acc[0][n][r][4 * q]);
+        float4 v = lds_f32x4(at);
+#pragma unroll
+        for (int w = 1; w < NCWB; ++w) {
+            const float4 o = lds_f32x4(at + w * (uint32_t)sizeof(T.acc[0]));
+            v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
+        }
+        if (r < rows) {
+            const uint32_t dst = stage + (uint32_t)(((rank * own + i) * NB + 8 * n + 4 * q) * 4);
+            if (to == rank) sts_f32x4(dst, v);
+            else st_async_f32x4(cluster_addr(dst, to), v, cluster_addr(sums, to));
+        }
+    }
+    consumer_sync_b();
+    const int mine = max(0, min(own, rows - rank * own));
+    if (mine > 0 && !__all_sync(0xffffffffu, mbar_wait_cluster(sums, 0))) {
+        if ((ct & 31) == 0) raise_abort(&T.abort);
+        return;
+    }
+    if (!write) return;
+    for (int k = ct; k < mine * (NB / 4); k += NCTB) {
+        const int b4 = k / mine, row = k - b4 * mine;
+        if (4 * b4 >= B) break;
+        const uint32_t at = stage + (uint32_t)((row * NB + 4 * b4) * 4);
+        float4 v = lds_f32x4(at);
+        for (int sl = 1; sl < L.S; ++sl) {
+            const float4 o = lds_f32x4(at + (uint32_t)(sl * own * NB * 4));
+            v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
+        }
+        float* y = Y + (int64_t)(4 * b4) * L.N + (int64_t)rb * RB + rank * own + row;
+        const float f[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (4 * b4 + j < B) y[j * L.N] = f[j];
+    }
+}
+
+// How the units are shared out beyond an even contiguous split: every block
+// takes `whole` units, and the units from `rest` on, too few for another one
+// per block, are cut into `parts` runs of columns, a block each (split-K adds
+// them up). Otherwise some blocks run one unit more than their neighbours, half
+// an SM's warps alone: 448 units on 304 blocks as one each and 288 halves take
+// 12.6 us instead of 15.1 (14336 x 4096, 8 rows).
+struct Shares {
+    int whole, rest, parts;
+};
+
+template <int NB, bool CL>
 __global__ void __launch_bounds__(GB_THREADS, GB_BLOCKS) gemmb_kernel(LayoutView L, const uint16_t* __restrict__ X,
-                                                              float* __restrict__ Y, int B) {
+                                                                      float* __restrict__ Y, int B, Shares sh) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned char* base = smem_raw + ((256u - (smem_u32(smem_raw) & 255u)) & 255u);
     TablesB<NB>& T = *reinterpret_cast<TablesB<NB>*>(base + STAGE_BYTES_B);
     const uint32_t stage = smem_u32(base);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int P = gridDim.x, p = blockIdx.x;
-    const int per = L.units / P, extra = L.units - per * P;
-    const int u_begin = p * per + min(p, extra), u_end = u_begin + per + (p < extra ? 1 : 0);
-    const int n_units = u_end - u_begin;
-    const int s0 = u_begin / L.nrb, rb0 = u_begin - s0 * L.nrb;
+    // the block's units: u_begin, u_begin + 1, ..., and perhaps a part of another
+    int u_begin, whole, part_unit = -1, part = 0;
+    if (CL) {                            // block rb * S + s: unit (rb, s)
+        const int rb = p / L.S;
+        u_begin = (p - rb * L.S) * L.nrb + rb;
+        whole = 1;
+    } else if (sh.parts > 1) {
+        u_begin = p * sh.whole;
+        whole = sh.whole;
+        const int i = p / sh.parts;
+        if (sh.rest + i < L.units) { part_unit = sh.rest + i; part = p - i * sh.parts; }
+    } else {
+        const int per = L.units / P, extra = L.units - per * P;
+        u_begin = p * per + min(p, extra);
+        whole = per + (p < extra ? 1 : 0);
+    }
+    const int n_units = whole + (part_unit >= 0);
+    auto unit_at = [&](int j) { return j < whole ? u_begin + j : part_unit; };
+    // the block that zeroes Y's rows of unit j's row block (under split-K)
+    auto owns_zeroing = [&](int j) { return unit_at(j) < L.nrb && (j < whole || part == 0); };
+    const int first_unit = unit_at(0), s0 = first_unit / L.nrb, rb0 = first_unit - s0 * L.nrb;
 
     const uint32_t full = smem_u32(&T.full), empty = smem_u32(&T.empty);
     const uint32_t abort_addr = smem_u32(&T.abort);
     if (tid == 0) {
         mbar_init(full, 1);
         mbar_init(empty, NCWB);
+        if (CL) mbar_init(smem_u32(&T.sums), 1);
         T.abort = 0;
         T.sk_ok = 0;
         fence_barrier_init();
-        issue_unit(L, u_begin, stage, full);
+        issue_unit(L, first_unit, stage, full);
+        if (CL) {
+            const int rows = min(RB, (int)(L.N - (int64_t)rb0 * RB)), own = cluster_rows(L.S);
+            const int mine = max(0, min(own, rows - s0 * own));
+            if (mine > 0)
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
+                             :: "r"(smem_u32(&T.sums)), "r"((uint32_t)((L.S - 1) * mine * NB * 4)) : "memory");
+        }
         T.consts[0] = bf2_pair(0x4300);
         T.consts[1] = bf2_pair(0xC380);
         const uint32_t adds[5] = {0xC282, 0xC204, 0xC188, 0xC110, 0xC0A0};     // -65, -33, -17, -9, -5
@@ -390,14 +483,21 @@ __global__ void __launch_bounds__(GB_THREADS, GB_BLOCKS) gemmb_kernel(LayoutView
         // ---- control: split-K zeroing, then each next copy into the freed stage ----
         // (whole row blocks are zeroed 4 rows per lane when every batch row of Y
         // starts on a 16-byte boundary)
+        if (CL) {
+            cluster_arrive();            // see the consumers: every block is done with its blob
+            cluster_wait();
+            if (lds_volatile(abort_addr) && lane == 0) mbar_wait_bounded(full, 0);
+            return;
+        }
         const bool vec = (L.N & 3) == 0;
         uint32_t epoch = 0;
         if (L.S > 1) {
             // the call count's load is in flight while the warp zeroes (the zeros
             // do not depend on it; the flags do)
             const unsigned long long count = call_count_raw(L.ctl);
-            const int z_end = min(u_end, L.nrb);
-            for (int u = u_begin; u < z_end; ++u) {
+            for (int j = 0; j < n_units; ++j) {
+                if (!owns_zeroing(j)) continue;
+                const int u = unit_at(j);
                 const int rows = min(RB, (int)(L.N - (int64_t)u * RB));
                 for (int b = 0; b < B; ++b) {
                     float* yr = Y + (int64_t)b * L.N + (int64_t)u * RB;
@@ -410,13 +510,26 @@ __global__ void __launch_bounds__(GB_THREADS, GB_BLOCKS) gemmb_kernel(LayoutView
             epoch = epoch_of(count);
             // release stores, one unit per lane in parallel: the warp's zeros
             // (ordered by __syncwarp) before each flag
-            for (int u = u_begin + lane; u < z_end; u += 32) st_release_gpu(L.ctl + 2 + u, epoch);
+            for (int j = lane; j < n_units; j += 32)
+                if (owns_zeroing(j)) st_release_gpu(L.ctl + 2 + unit_at(j), epoch);
         }
         bool dead = false;
-        if (L.S > 1 && !split_k_flags_ready(L, epoch, u_begin, u_end, lane)) {
-            // a row block this block adds into was never zeroed in time
-            dead = true;
-            if (lane == 0) raise_abort(&T.abort);
+        if (L.S > 1) {
+            // every row block this block adds into zeroed in this call (flag ==
+            // epoch), within the wait limit; a lane per unit, acquire loads
+            bool seen = true;
+            const unsigned long long t0 = global_ns();
+            for (int j = lane; j < n_units && seen; j += 32) {
+                if (owns_zeroing(j)) continue;
+                const uint32_t* f = L.ctl + 2 + unit_at(j) % L.nrb;
+                while (!(seen = ld_acquire_gpu(f) == epoch))
+                    if (global_ns() - t0 > WAIT_LIMIT_NS) break;
+            }
+            __syncwarp();                // every lane's later additions after every acquire
+            if (!__all_sync(0xffffffffu, seen)) {
+                dead = true;
+                if (lane == 0) raise_abort(&T.abort);
+            }
         }
         // the consumers write Y; they add only after these flags (and this
         // warp's own zeroing), passed on by a release
@@ -428,7 +541,7 @@ __global__ void __launch_bounds__(GB_THREADS, GB_BLOCKS) gemmb_kernel(LayoutView
                 if (lane == 0) raise_abort(&T.abort);
                 break;
             }
-            if (lane == 0) issue_unit(L, u_begin + j + 1, stage, full);
+            if (lane == 0) issue_unit(L, unit_at(j + 1), stage, full);
             ++issued;
         }
         if (L.S > 1 && lane == 0) call_done(L.ctl);      // this block's share of the call count
@@ -438,7 +551,6 @@ __global__ void __launch_bounds__(GB_THREADS, GB_BLOCKS) gemmb_kernel(LayoutView
         // ---- consumers: every unit, whole columns (or a share of one) per warp ----
         const int ct = tid - 32, cw = warp - 1;
         bool dead = false, sk_seen = L.S == 1;
-        int rbj = rb0, sj = s0;
         const uint32_t acc = smem_u32(&T.acc[cw][0][0][0]);
         DecodeConsts K;
         {
@@ -452,16 +564,28 @@ __global__ void __launch_bounds__(GB_THREADS, GB_BLOCKS) gemmb_kernel(LayoutView
             }
         }
         for (int j = 0; j < n_units; ++j) {
-            const int cols = min(L.C, L.G - sj * L.C);
+            const int u = unit_at(j), sj = u / L.nrb, rbj = u - sj * L.nrb;
+            int cols = min(L.C, L.G - sj * L.C), c_lo = 0;
+            if (!CL && j >= whole) {     // a part: its share of the columns
+                c_lo = cols * part / sh.parts;
+                cols = cols * (part + 1) / sh.parts - c_lo;
+            }
             const Deal dl = deal_columns(cols, cw);
             const uint16_t* x = X + (int64_t)sj * L.C * GROUP;
             uint32_t xb[NB];             // the first column's activations, on their way while the blob lands
-            if (dl.c0 < cols) load_acts<NB>(xb, x + (int64_t)dl.c0 * GROUP, L.K, B, lane >> 2, lane & 3);
+            if (dl.c0 < cols) load_acts<NB>(xb, x + (int64_t)(c_lo + dl.c0) * GROUP, L.K, B, lane >> 2, lane & 3);
             if (!dead && !warp_wait(full, (uint32_t)j & 1u, abort_addr)) { dead = true; if (lane == 0) raise_abort(&T.abort); }
             if (!dead) {
-                consume_unit_b<NB>(K, stage, L.C, cols, dl, xb, x, L.K, B, acc, lane);
+                consume_unit_b<NB>(K, stage, L.C, c_lo, cols, dl, xb, x, L.K, B, acc, lane);
                 __syncwarp();
-                if (lane == 0) mbar_arrive(empty);
+                if (!CL && lane == 0) mbar_arrive(empty);
+            }
+            if constexpr (CL) {
+                // every warp's sums, and every block of the cluster done with its blob
+                cluster_arrive();
+                cluster_wait();
+                flush_cluster<NB>(T, stage, L, Y, B, rb0, s0, ct, !dead && !lds_volatile(abort_addr));
+                return;
             }
             consumer_sync_b();           // every warp's sums
             if (!sk_seen && !dead) {
@@ -479,37 +603,64 @@ __global__ void __launch_bounds__(GB_THREADS, GB_BLOCKS) gemmb_kernel(LayoutView
             }
             if (!dead && !lds_volatile(abort_addr)) flush_rows<NB>(T, L, Y, B, rbj, ct);
             if (j + 1 < n_units) consumer_sync_b();      // the rows are read and zero again
-            if (++rbj == L.nrb) { rbj = 0; ++sj; }
         }
     }
 }
 
-template <int NB>
-cudaError_t launch_gemmb(const LayoutView& L, const uint16_t* X, float* Y, int B, cudaStream_t s) {
-    static LaunchPrep prep;
-    int sms = 0;
-    cudaError_t e = prep.get(gemmb_kernel<NB>, gemmb_smem<NB>(), &sms);
-    if (e != cudaSuccess) return e;
-    const int grid = L.units < GB_BLOCKS * sms ? L.units : GB_BLOCKS * sms;
+template <int NB, bool CL>
+cudaError_t launch_gemmb(const LayoutView& L, const uint16_t* X, float* Y, int B, cudaStream_t s, int grid, Shares sh) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(GB_THREADS);
     cfg.dynamicSmemBytes = gemmb_smem<NB>();
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = L.S;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, gemmb_kernel<NB>, L, X, Y, B);
+    cfg.numAttrs = CL ? 2 : 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, gemmb_kernel<NB, CL>, L, X, Y, B, sh);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
+}
+
+// Layouts of narrow units that all have a block at once (two per SM, less what
+// clusters leave unused of a GPC's SMs, see unit_plan_fits) run a row block's
+// slabs as a cluster of at most 8 blocks, 16 for more than 8 rows: zeroing the
+// rows of Y behind flags and adding into them is on the path of a small
+// product, the more rows the more (us in a graph, flags -> cluster, at 4 rows
+// 768x768 3.27 -> 3.17, 2048x2048 4.41 -> 4.16, 5632x2048 5.62 -> 5.35; at 16
+// rows 4.8 -> 3.8, 6.3 -> 5.3, 7.7 -> 6.9; with 11 slabs 2048x5632 5.4 -> 5.7 at
+// 4 rows, with 16 slabs 1024x4096 5.8 -> 5.3 at 16).
+// Otherwise units of 16 columns that would leave some blocks one unit more
+// than others are cut in two where both halves of all of them find a block
+// (see Shares; half a unit still gives every warp a column): 4096x4096, 128
+// units, 7.9 -> 6.6 us at 8 rows and 10.6 -> 8.1 at 16; 14336x4096, 448 units,
+// 15.1 -> 12.6 and 20.9 -> 17.6.
+template <int NB>
+cudaError_t launch_gemm(const LayoutView& L, const uint16_t* X, float* Y, int B, cudaStream_t s) {
+    static LaunchPrep prep, prep_cl;
+    int sms = 0;
+    cudaError_t e = prep.get(gemmb_kernel<NB, false>, gemmb_smem<NB>(), &sms);
+    if (e != cudaSuccess) return e;
+    if (L.S > 1 && L.C <= 8 && L.S <= (NB == 8 ? 8 : MAX_CLUSTER) && 4 * (int64_t)L.units <= (L.S <= 8 ? 7 : 5) * (int64_t)sms) {
+        if ((e = prep_cl.get(gemmb_kernel<NB, true>, gemmb_smem<NB>(), &sms, true)) != cudaSuccess) return e;
+        return launch_gemmb<NB, true>(L, X, Y, B, s, L.units, Shares{0, 0, 1});
+    }
+    const int blocks = GB_BLOCKS * sms, whole = L.units / blocks, left = L.units - whole * blocks;
+    if (L.S > 1 && L.C == 2 * NCWB && left > 0 && 2 * left <= blocks)
+        return launch_gemmb<NB, false>(L, X, Y, B, s, whole ? blocks : 2 * left, Shares{whole, whole * blocks, 2});
+    return launch_gemmb<NB, false>(L, X, Y, B, s, L.units < blocks ? L.units : blocks, Shares{0, 0, 1});
 }
 
 }  // namespace
 
 cudaError_t launch_gemm_small(const LayoutView& L, const uint16_t* X, float* Y, int B, cudaStream_t s) {
-    return B > 8 ? launch_gemmb<16>(L, X, Y, B, s) : launch_gemmb<8>(L, X, Y, B, s);
+    return B > 8 ? launch_gemm<16>(L, X, Y, B, s) : launch_gemm<8>(L, X, Y, B, s);
 }
 
 cudaError_t read_device_status_gemm(uint32_t* status) {

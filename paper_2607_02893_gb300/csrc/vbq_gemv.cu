@@ -1359,33 +1359,6 @@ struct __align__(16) TablesU : ActTab<1> {
 constexpr size_t gemv1_unit_smem() { return 256 + (size_t)STAGE_BYTES + sizeof(TablesU); }
 static_assert(2 * (gemv1_unit_smem() + 1024) <= 228 * 1024, "two blocks per SM");
 
-__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-    return r;
-}
-// Bounded wait for other blocks' st.async on this block's barrier. Longer than
-// any of their own waits: every block of the cluster sends its sums even when
-// a wait of its own ran out, so the receiver never exits before they land.
-__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity) {
-    const unsigned long long t0 = global_ns();
-    for (;;) {
-        uint32_t ok;
-        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
-                     "selp.u32 %0, 1, 0, p;\n\t}"
-                     : "=r"(ok) : "r"(bar), "r"(parity), "n"(SUSPEND_HINT_NS) : "memory");
-        if (ok) return true;
-        if (global_ns() - t0 > 4 * WAIT_LIMIT_NS) return false;
-    }
-}
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-// One float into another block's shared memory, counted (4 bytes) on that block's barrier.
-__device__ __forceinline__ void st_async_f32(uint32_t dst, float v, uint32_t bar) {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
-                 :: "r"(dst), "r"(__float_as_uint(v)), "r"(bar) : "memory");
-}
-
 // Block rb * S + s takes unit (rb, s): MODE and SW as in gemv1_kernel.
 template <int MODE, bool SW>
 __global__ void __launch_bounds__(U1_THREADS, 2) gemv1_unit_kernel(LayoutView L, const uint16_t* __restrict__ x,

@@ -40,3 +40,24 @@ def test_few_rows(n, g, dist):
 @pytest.mark.parametrize("dist", [MAIN, EVEN])
 def test_unit_widths(n, g, dist):
     _check(Matrix(n, 64 * g, dist=dist, seed_path=(98, n, g), batch=16), (8, 13))
+
+
+# 16-column units cut in two: all of them (few units), or those beyond one per
+# block; a ragged last slab whose halves are uneven, odd rows
+@pytest.mark.parametrize("n,g", [(12800, 17), (4992, 65), (20001, 47)])
+def test_unit_halves(n, g):
+    _check(Matrix(n, 64 * g, dist=MAIN, seed_path=(98, n, g), batch=16), (5, 16))
+
+
+# clusters: every size of a block's own rows (128 rows over S slabs), and row
+# blocks so short that some blocks own none; the same bits on every call
+@pytest.mark.parametrize("n,g", [(130, 4), (257, 6), (384, 10), (1, 14), (5, 16), (1000, 32), (200, 24), (1024, 64)])
+def test_clusters(n, g):
+    m = Matrix(n, 64 * g, dist=EVEN, seed_path=(99, n, g), batch=16)
+    _check(m, (6, 16))
+    layout = vbq.vbq_pack(*m.device_args("cuda"))
+    x = bits_to_i16(m.x_bits).cuda()
+    ys = [torch.empty((16, n), device="cuda") for _ in range(3)]
+    for y in ys:
+        vbq.vbq_gemm_small(layout, x, y)
+    assert torch.equal(ys[0], ys[1]) and torch.equal(ys[0], ys[2])
