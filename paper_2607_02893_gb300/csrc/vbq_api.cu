@@ -65,7 +65,10 @@ struct TempBuffers {
 // those allocates its own.
 class ErrorWords {
 public:
+    // The words may be another call's next: a kernel of this one that has not
+    // been synchronised with (an error on the way out) is waited for first.
     ~ErrorWords() {
+        if (armed_) cudaStreamSynchronize(stream_);
         if (slot_ >= 0) {
             std::lock_guard<std::mutex> lock(mu_);
             used_ &= ~(1ull << slot_);
@@ -73,7 +76,8 @@ public:
             cudaFreeHost(w_);
         }
     }
-    cudaError_t get() {
+    cudaError_t get(cudaStream_t stream) {
+        stream_ = stream;
         {
             std::lock_guard<std::mutex> lock(mu_);
             if (!page_) {
@@ -94,7 +98,15 @@ public:
         w_[0] = w_[1] = 0;
         return cudaSuccess;
     }
-    uint32_t* word(int i) const { return w_ + i; }
+    uint32_t* arm(int i) {                  // for a kernel about to be launched on the stream
+        armed_ = true;
+        return w_ + i;
+    }
+    cudaError_t settle() {                  // wait for the stream; the words can be read
+        const cudaError_t e = cudaStreamSynchronize(stream_);
+        armed_ = false;
+        return e;
+    }
     bool set(int i) const { return static_cast<volatile uint32_t*>(w_)[i] != 0; }
 
 private:
@@ -106,6 +118,8 @@ private:
     static uint64_t used_;
     uint32_t* w_ = nullptr;
     int slot_ = -1;
+    cudaStream_t stream_ = nullptr;
+    bool armed_ = false;
 };
 std::mutex ErrorWords::mu_;
 uint32_t* ErrorWords::page_ = nullptr;
@@ -184,7 +198,7 @@ vbq_status_t vbq_pack(const uint8_t* codes, const uint8_t* bitwidths, const uint
     const size_t ncodes = (size_t)N * (size_t)K, ngroups = (size_t)N * (size_t)G;
     TempBuffers tmp;
     ErrorWords err;
-    VBQ_CUDA(err.get());
+    VBQ_CUDA(err.get(s));
 
     const uint8_t* d_codes = codes;
     const uint8_t* d_widths = bitwidths;
@@ -246,9 +260,9 @@ vbq_status_t vbq_pack(const uint8_t* codes, const uint8_t* bitwidths, const uint
         std::vector<uint32_t> cnt((size_t)uc * 5);
         VBQ_CUDA(tmp.alloc(&dc, cnt.size() * sizeof(uint32_t)));
         d_counts = static_cast<uint32_t*>(dc);
-        VBQ_CUDA(vbq::launch_count(d_widths, N, (int)G, cand, (int)nrb, (int)uc, d_counts, err.word(0), s));
+        VBQ_CUDA(vbq::launch_count(d_widths, N, (int)G, cand, (int)nrb, (int)uc, d_counts, err.arm(0), s));
         VBQ_CUDA(cudaMemcpyAsync(cnt.data(), dc, cnt.size() * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-        VBQ_CUDA(cudaStreamSynchronize(s));
+        VBQ_CUDA(err.settle());
         if (err.set(0)) return fail(VBQ_ERR_WIDTH, "a bit-width is not in {1,2,4,8}");
         std::vector<uint32_t> size16((size_t)uc);
         uint32_t m16 = 0;
@@ -329,9 +343,9 @@ vbq_status_t vbq_pack(const uint8_t* codes, const uint8_t* bitwidths, const uint
     if ((e = cudaMemcpyAsync(base + off_at, blob_off.data(), blob_off.size() * 4, cudaMemcpyHostToDevice, s)) !=
         cudaSuccess)
         return bail(VBQ_ERR_CUDA, "offset copy", e);
-    if ((e = vbq::launch_scatter(d_codes, d_widths, d_scales, d_counts, V, base, err.word(1), s)) != cudaSuccess)
+    if ((e = vbq::launch_scatter(d_codes, d_widths, d_scales, d_counts, V, base, err.arm(1), s)) != cudaSuccess)
         return bail(VBQ_ERR_CUDA, "scatter launch", e);
-    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return bail(VBQ_ERR_CUDA, "pack", e);
+    if ((e = err.settle()) != cudaSuccess) return bail(VBQ_ERR_CUDA, "pack", e);
     if (err.set(1)) {
         cudaFree(L->base);
         delete L;
@@ -371,9 +385,9 @@ vbq_status_t vbq_quantize(const float* w, const uint8_t* bitwidths, int64_t N, i
         return fail(VBQ_ERR_ALIGN, "device arrays must be 16-byte aligned");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     ErrorWords err;
-    VBQ_CUDA(err.get());
-    VBQ_CUDA(vbq::launch_quant_validate(w, bitwidths, N, K, err.word(0), s));
-    VBQ_CUDA(cudaStreamSynchronize(s));
+    VBQ_CUDA(err.get(s));
+    VBQ_CUDA(vbq::launch_quant_validate(w, bitwidths, N, K, err.arm(0), s));
+    VBQ_CUDA(err.settle());
     if (err.set(0)) return fail(VBQ_ERR_WIDTH, "a bit-width is not in {1,2,4,8}");
     if (err.set(1)) return fail(VBQ_ERR_ARG, "a weight is NaN");
     VBQ_CUDA(vbq::launch_quantize(w, bitwidths, N, K, codes_out, scales_out, s));
