@@ -324,6 +324,7 @@ __device__ __forceinline__ void flush_rows(TablesB<NB>& T, const LayoutView& L, 
 #pragma unroll
     for (int n = 0; n < NB / 8; ++n) {
         const int b0 = 8 * n + 4 * q;
+        if (b0 >= B) continue;           // absent batch rows: their sums stay zero
         const uint32_t at = smem_u32(&T.acc[0][n][r][4 * q]);
         float4 v = lds_f32x4(at);
         sts_zero4(at);
@@ -357,6 +358,7 @@ __device__ __forceinline__ void flush_rows(TablesB<NB>& T, const LayoutView& L, 
 // bits on every call. Slab k's sums of a block's row i sit at ((k * own + i) *
 // NB) floats. write is false after a wait that ran out.
 __host__ __device__ inline int cluster_rows(int S) { return (RB + S - 1) / S; }
+__host__ __device__ inline int batch_quads(int B) { return (B + 3) / 4; }      // only these batch rows are exchanged
 template <int NB>
 __device__ __forceinline__ void flush_cluster(TablesB<NB>& T, uint32_t stage, const LayoutView& L, float* __restrict__ Y, int B,
                                               int rb, int rank, int ct, bool write) {
@@ -365,6 +367,7 @@ __device__ __forceinline__ void flush_cluster(TablesB<NB>& T, uint32_t stage, co
     const int r = ct >> 1, q = ct & 1, to = r / own, i = r - to * own;
 #pragma unroll
     for (int n = 0; n < NB / 8; ++n) {
+        if (8 * n + 4 * q >= B) continue;
         const uint32_t at = smem_u32(&T.acc[0][n][r][4 * q]);
         float4 v = lds_f32x4(at);
 #pragma unroll
@@ -385,9 +388,8 @@ __device__ __forceinline__ void flush_cluster(TablesB<NB>& T, uint32_t stage, co
         return;
     }
     if (!write) return;
-    for (int k = ct; k < mine * (NB / 4); k += NCTB) {
+    for (int k = ct; k < mine * batch_quads(B); k += NCTB) {
         const int b4 = k / mine, row = k - b4 * mine;
-        if (4 * b4 >= B) break;
         const uint32_t at = stage + (uint32_t)((row * NB + 4 * b4) * 4);
         float4 v = lds_f32x4(at);
         for (int sl = 1; sl < L.S; ++sl) {
@@ -458,7 +460,7 @@ __global__ void __launch_bounds__(GB_THREADS, GB_BLOCKS) gemmb_kernel(LayoutView
             const int mine = max(0, min(own, rows - s0 * own));
             if (mine > 0)
                 asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
-                             :: "r"(smem_u32(&T.sums)), "r"((uint32_t)((L.S - 1) * mine * NB * 4)) : "memory");
+                             :: "r"(smem_u32(&T.sums)), "r"((uint32_t)((L.S - 1) * mine * batch_quads(B) * 16)) : "memory");
         }
         T.consts[0] = bf2_pair(0x4300);
         T.consts[1] = bf2_pair(0xC380);

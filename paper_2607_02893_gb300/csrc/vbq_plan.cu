@@ -9,15 +9,15 @@ namespace vbq {
 // whichever the layout's width mix makes cheaper. Cost per million groups of
 // each width (1, 2, 4, 8 bits), in microseconds, measured on a GB300 on
 // 16384 x 16384 matrices of one width: one row on the table kernel, two rows
-// on it, and up to 8 rows on the tensor cores. The tensor cores take items in
+// on it, and four rows on the tensor cores. The tensor cores take items in
 // tiles of 16 from each (column, width) bucket of a unit, so a bucket leaves
-// about 6 item slots of its last tile idle (16384 x 16384 of the main mix at 8
-// rows: 57 us measured, 57 us modelled). So two rows of a 1- or 2-bit heavy
-// matrix stay on the tables (main mix 42 against 57 us) and three or four go
-// to the tensor cores (64 and 83 against 57 us).
+// about 6 item slots of its last tile idle (16384 x 16384 of the main mix: 50
+// us measured at 4 rows, 55 us modelled). So two rows of a 1- or 2-bit heavy
+// matrix stay on the tables (main mix 43 us) and three or four go to the
+// tensor cores (64 and 83 us on the tables).
 constexpr double COST_ONE[4] = {4.09, 5.86, 8.78, 13.1};
-constexpr double COST_PAIR[4] = {8.06, 10.8, 15.9, 19.9};
-constexpr double COST_MMA[4] = {9.78, 10.9, 13.4, 22.5};
+constexpr double COST_PAIR[4] = {8.06, 10.8, 15.9, 24.0};
+constexpr double COST_MMA[4] = {9.3, 10.4, 12.7, 20.8};
 constexpr double MMA_IDLE_PER_BUCKET = 6.0;
 
 bool tables_for_batch(const LayoutView& L, int B) {
