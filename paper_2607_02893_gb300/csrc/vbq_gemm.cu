@@ -632,12 +632,14 @@ cudaError_t launch_gemmb(const LayoutView& L, const uint16_t* X, float* Y, int B
 
 // Layouts of narrow units that all have a block at once (two per SM, less what
 // clusters leave unused of a GPC's SMs, see unit_plan_fits) run a row block's
-// slabs as a cluster of at most 8 blocks, 16 for more than 8 rows: zeroing the
-// rows of Y behind flags and adding into them is on the path of a small
-// product, the more rows the more (us in a graph, flags -> cluster, at 4 rows
-// 768x768 3.27 -> 3.17, 2048x2048 4.41 -> 4.16, 5632x2048 5.62 -> 5.35; at 16
-// rows 4.8 -> 3.8, 6.3 -> 5.3, 7.7 -> 6.9; with 11 slabs 2048x5632 5.4 -> 5.7 at
-// 4 rows, with 16 slabs 1024x4096 5.8 -> 5.3 at 16).
+// slabs as a cluster for more than 8 rows, and for 5 to 8 where the matrix, and
+// a square one on its input (its neighbours on the stream), is small (under
+// 50,000 groups, at most 8 slabs): zeroing the rows of Y behind flags and adding
+// into them is then on the product's path. Flags -> cluster (us in a graph): at
+// 16 rows 768x768 4.8 -> 3.8, 2048x2048 6.3 -> 5.3, 1024x4096 5.8 -> 5.3; four ~131M
+// layers at 8 rows 107.7 -> 101.1, at 4 rows 98.6 -> 98.0, at 3 rows 95.9 -> 97.1;
+// a ~1B layer (16,384 to 180,224 groups a product) at 4 rows 34.2 -> 36.2, at 6
+// rows 35.3 -> 36.7 with all of it as clusters and 38.7 with the smallest alone.
 // Otherwise units of 16 columns that would leave some blocks one unit more
 // than others are cut in two where both halves of all of them find a block
 // (see Shares; half a unit still gives every warp a column): 4096x4096, 128
@@ -649,7 +651,10 @@ cudaError_t launch_gemm(const LayoutView& L, const uint16_t* X, float* Y, int B,
     int sms = 0;
     cudaError_t e = prep.get(gemmb_kernel<NB, false>, gemmb_smem<NB>(), &sms);
     if (e != cudaSuccess) return e;
-    if (L.S > 1 && L.C <= 8 && L.S <= (NB == 8 ? 8 : MAX_CLUSTER) && 4 * (int64_t)L.units <= (L.S <= 8 ? 7 : 5) * (int64_t)sms) {
+    constexpr int64_t SMALL = 50000;
+    const bool pays = NB == 16 ? L.S <= MAX_CLUSTER
+                               : B > 4 && L.S <= 8 && L.N * L.G < SMALL && GROUP * (int64_t)L.G * L.G < SMALL;
+    if (pays && L.S > 1 && L.C <= 8 && 4 * (int64_t)L.units <= (L.S <= 8 ? 7 : 5) * (int64_t)sms) {
         if ((e = prep_cl.get(gemmb_kernel<NB, true>, gemmb_smem<NB>(), &sms, true)) != cudaSuccess) return e;
         return launch_gemmb<NB, true>(L, X, Y, B, s, L.units, Shares{0, 0, 1});
     }
