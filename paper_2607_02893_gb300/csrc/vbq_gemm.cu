@@ -30,7 +30,7 @@
 // product in a graph of dependent products, before -> now: 14336 x 4096 main
 // 18.6 -> 12.6 us at 8 rows and 34.7 -> 17.6 at 16; 16384^2 all 1 bit 59 -> 42
 // and 97 -> 63, all 2 bits 71 -> 46 and 106 -> 64, all 4 bits 72 -> 58 and 121
-// -> 84, all 8 bits 98 -> 97 and 170 -> 136. The error against 64 bits fell
+// -> 83, all 8 bits 98 -> 97 and 170 -> 136. The error against 64 bits fell
 // from 5e-6 to 1e-7 of the result's norm: denormal operands lose their
 // alignment in the tensor core's sums, normal bf16 ones do not.
 //
