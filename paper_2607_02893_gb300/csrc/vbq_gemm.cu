@@ -44,6 +44,7 @@
 // and each 128-item tile costs its warps about 200 instructions of waits,
 // fences and issue; 14336 x 4096 main at 8 rows took 25 us.)
 #include "vbq_kernels.h"
+#include "vbq_deal.h"
 #include "vbq_device.cuh"
 #include <cuda_bf16.h>
 
@@ -404,16 +405,6 @@ __device__ __forceinline__ void flush_cluster(TablesB<NB>& T, uint32_t stage, co
     }
 }
 
-// How the units are shared out beyond an even contiguous split: every block
-// takes `whole` units, and the units from `rest` on, too few for another one
-// per block, are cut into `parts` runs of columns, a block each (split-K adds
-// them up). Otherwise some blocks run one unit more than their neighbours, half
-// an SM's warps alone: 448 units on 304 blocks as one each and 288 halves take
-// 12.6 us instead of 15.1 (14336 x 4096, 8 rows).
-struct Shares {
-    int whole, rest, parts;
-};
-
 template <int NB, bool CL>
 __global__ void __launch_bounds__(GB_THREADS, GB_BLOCKS) gemmb_kernel(LayoutView L, const uint16_t* __restrict__ X,
                                                                       float* __restrict__ Y, int B, Shares sh) {
@@ -423,27 +414,26 @@ __global__ void __launch_bounds__(GB_THREADS, GB_BLOCKS) gemmb_kernel(LayoutView
     const uint32_t stage = smem_u32(base);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int P = gridDim.x, p = blockIdx.x;
-    // the block's units: u_begin, u_begin + 1, ..., and perhaps a part of another
-    int u_begin, whole, part_unit = -1, part = 0;
+    // the block's places in the deal: begin, begin + 1, ..., and perhaps a part of another
+    int begin, whole, part_at = -1, part = 0;
     if (CL) {                            // block rb * S + s: unit (rb, s)
         const int rb = p / L.S;
-        u_begin = (p - rb * L.S) * L.nrb + rb;
+        begin = (p - rb * L.S) * L.nrb + rb;
         whole = 1;
-    } else if (sh.parts > 1) {
-        u_begin = p * sh.whole;
-        whole = sh.whole;
-        const int i = p / sh.parts;
-        if (sh.rest + i < L.units) { part_unit = sh.rest + i; part = p - i * sh.parts; }
     } else {
-        const int per = L.units / P, extra = L.units - per * P;
-        u_begin = p * per + min(p, extra);
-        whole = per + (p < extra ? 1 : 0);
+        const BlockShare b = block_share(L.units, sh, P, p);
+        begin = b.begin;
+        whole = b.whole;
+        part_at = b.part_at;
+        part = b.part;
     }
-    const int n_units = whole + (part_unit >= 0);
-    auto unit_at = [&](int j) { return j < whole ? u_begin + j : part_unit; };
-    // the block that zeroes Y's rows of unit j's row block (under split-K)
-    auto owns_zeroing = [&](int j) { return unit_at(j) < L.nrb && (j < whole || part == 0); };
-    const int first_unit = unit_at(0), s0 = first_unit / L.nrb, rb0 = first_unit - s0 * L.nrb;
+    const int n_units = whole + (part_at >= 0), rot = CL ? 0 : sh.rot;
+    auto place = [&](int j) { return j < whole ? begin + j : part_at; };
+    // the block that zeroes Y's rows of place j's row block (under split-K; slab 0 is dealt in order)
+    auto owns_zeroing = [&](int j) { return place(j) < L.nrb && (j < whole || part == 0); };
+    auto row_block = [&](int j) { return dealt_row_block(place(j), place(j) / L.nrb, L.nrb, rot); };
+    const int rb_lane = lane < n_units ? row_block(lane) : 0;      // a division, ahead of the wait
+    const int s0 = place(0) / L.nrb, rb0 = dealt_row_block(place(0), s0, L.nrb, rot);
 
     const uint32_t full = smem_u32(&T.full), empty = smem_u32(&T.empty);
     const uint32_t abort_addr = smem_u32(&T.abort);
@@ -454,7 +444,7 @@ __global__ void __launch_bounds__(GB_THREADS, GB_BLOCKS) gemmb_kernel(LayoutView
         T.abort = 0;
         T.sk_ok = 0;
         fence_barrier_init();
-        issue_unit(L, first_unit, stage, full);
+        issue_unit(L, s0 * L.nrb + rb0, stage, full);
         if (CL) {
             const int rows = min(RB, (int)(L.N - (int64_t)rb0 * RB)), own = cluster_rows(L.S);
             const int mine = max(0, min(own, rows - s0 * own));
@@ -499,7 +489,7 @@ __global__ void __launch_bounds__(GB_THREADS, GB_BLOCKS) gemmb_kernel(LayoutView
             const unsigned long long count = call_count_raw(L.ctl);
             for (int j = 0; j < n_units; ++j) {
                 if (!owns_zeroing(j)) continue;
-                const int u = unit_at(j);
+                const int u = place(j);
                 const int rows = min(RB, (int)(L.N - (int64_t)u * RB));
                 for (int b = 0; b < B; ++b) {
                     float* yr = Y + (int64_t)b * L.N + (int64_t)u * RB;
@@ -513,7 +503,7 @@ __global__ void __launch_bounds__(GB_THREADS, GB_BLOCKS) gemmb_kernel(LayoutView
             // release stores, one unit per lane in parallel: the warp's zeros
             // (ordered by __syncwarp) before each flag
             for (int j = lane; j < n_units; j += 32)
-                if (owns_zeroing(j)) st_release_gpu(L.ctl + 2 + unit_at(j), epoch);
+                if (owns_zeroing(j)) st_release_gpu(L.ctl + 2 + place(j), epoch);
         }
         bool dead = false;
         if (L.S > 1) {
@@ -523,7 +513,7 @@ __global__ void __launch_bounds__(GB_THREADS, GB_BLOCKS) gemmb_kernel(LayoutView
             const unsigned long long t0 = global_ns();
             for (int j = lane; j < n_units && seen; j += 32) {
                 if (owns_zeroing(j)) continue;
-                const uint32_t* f = L.ctl + 2 + unit_at(j) % L.nrb;
+                const uint32_t* f = L.ctl + 2 + (j == lane ? rb_lane : row_block(j));
                 while (!(seen = ld_acquire_gpu(f) == epoch))
                     if (global_ns() - t0 > WAIT_LIMIT_NS) break;
             }
@@ -543,7 +533,10 @@ __global__ void __launch_bounds__(GB_THREADS, GB_BLOCKS) gemmb_kernel(LayoutView
                 if (lane == 0) raise_abort(&T.abort);
                 break;
             }
-            if (lane == 0) issue_unit(L, unit_at(j + 1), stage, full);
+            if (lane == 0) {
+                const int d = place(j + 1), sl = d / L.nrb;
+                issue_unit(L, sl * L.nrb + dealt_row_block(d, sl, L.nrb, rot), stage, full);
+            }
             ++issued;
         }
         if (L.S > 1 && lane == 0) call_done(L.ctl);      // this block's share of the call count
@@ -566,7 +559,7 @@ __global__ void __launch_bounds__(GB_THREADS, GB_BLOCKS) gemmb_kernel(LayoutView
             }
         }
         for (int j = 0; j < n_units; ++j) {
-            const int u = unit_at(j), sj = u / L.nrb, rbj = u - sj * L.nrb;
+            const int d = place(j), sj = d / L.nrb, rbj = dealt_row_block(d, sj, L.nrb, rot);
             int cols = min(L.C, L.G - sj * L.C), c_lo = 0;
             if (!CL && j >= whole) {     // a part: its share of the columns
                 c_lo = cols * part / sh.parts;
@@ -656,12 +649,11 @@ cudaError_t launch_gemm(const LayoutView& L, const uint16_t* X, float* Y, int B,
                                : B > 4 && L.S <= 8 && L.N * L.G < SMALL && GROUP * (int64_t)L.G * L.G < SMALL;
     if (pays && L.S > 1 && L.C <= 8 && 4 * (int64_t)L.units <= (L.S <= 8 ? 7 : 5) * (int64_t)sms) {
         if ((e = prep_cl.get(gemmb_kernel<NB, true>, gemmb_smem<NB>(), &sms, true)) != cudaSuccess) return e;
-        return launch_gemmb<NB, true>(L, X, Y, B, s, L.units, Shares{0, 0, 1});
+        return launch_gemmb<NB, true>(L, X, Y, B, s, L.units, Shares{0, 0, 1, 0});
     }
-    const int blocks = GB_BLOCKS * sms, whole = L.units / blocks, left = L.units - whole * blocks;
-    if (L.S > 1 && L.C == 2 * NCWB && left > 0 && 2 * left <= blocks)
-        return launch_gemmb<NB, false>(L, X, Y, B, s, whole ? blocks : 2 * left, Shares{whole, whole * blocks, 2});
-    return launch_gemmb<NB, false>(L, X, Y, B, s, L.units < blocks ? L.units : blocks, Shares{0, 0, 1});
+    const int blocks = GB_BLOCKS * sms;
+    const Shares sh = plan_shares(L.units, L.nrb, L.S, L.C == 2 * NCWB, blocks);
+    return launch_gemmb<NB, false>(L, X, Y, B, s, grid_blocks(L.units, sh, blocks), sh);
 }
 
 }  // namespace
