@@ -51,6 +51,14 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// Reads of shared memory come in two forms. To the compiler the plain ones are
+// functions of their address alone, which it may move or merge; the ordered ones
+// stay in their place among barriers, waits and other ordered accesses. A value
+// that some barrier, wait or earlier store of the block separates from another
+// value at the same address (a unit's header and task descriptors, column ends,
+// row sums, slots) is read in the ordered form. The plain form is for what such
+// a read leads to: addresses taken from a header or a descriptor, and tables at
+// columns taken from one, which cannot be known before it.
 template <int OFF>
 __device__ __forceinline__ float lds_f32(uint32_t addr) {
     float v;
@@ -74,6 +82,34 @@ __device__ __forceinline__ float4 lds_f32x4(uint32_t addr) {
     float4 v;
     asm("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
                  : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
+    return v;
+}
+
+__device__ __forceinline__ float4 lds_f32x4_ordered(uint32_t addr) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ float2 lds_f32x2_ordered(uint32_t addr) {
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint4 lds_u32x4_ordered(uint32_t addr) {
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t lds_u32_ordered(uint32_t addr) {
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t lds_u16_ordered(uint32_t addr) {
+    uint32_t v;
+    asm volatile("ld.shared.u16 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
     return v;
 }
 

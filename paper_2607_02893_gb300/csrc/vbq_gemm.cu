@@ -95,11 +95,6 @@ __device__ __forceinline__ void sts_f32x2(uint32_t addr, float2 v) {
 __device__ __forceinline__ void sts_f32x4(uint32_t addr, float4 v) {
     asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" :: "r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
 }
-__device__ __forceinline__ float2 lds_f32x2_ordered(uint32_t addr) {
-    float2 v;
-    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
-    return v;
-}
 
 // ---- levels as bf16 pairs -----------------------------------------------------
 //
@@ -285,15 +280,15 @@ __device__ __forceinline__ void consume_unit_b(const DecodeConsts& K, uint32_t s
                                                uint32_t (&xb)[NB], const uint16_t* __restrict__ x, int64_t Kx, int B,
                                                uint32_t acc, int lane) {
     const int g = lane >> 2, t = lane & 3, sh = 8 * (t & 1);
-    const uint4 h0 = lds_u32x4(sblob), h1 = lds_u32x4(sblob + 16), h2 = lds_u32x4(sblob + 32);
+    const uint4 h0 = lds_u32x4_ordered(sblob), h1 = lds_u32x4_ordered(sblob + 16), h2 = lds_u32x4_ordered(sblob + 32);
     const uint32_t cc = sblob + (h2.x & 0xFFFF) * 16;
     const uint32_t my = acc + 8u * t;
     for (int c = c_lo + dl.c0; c < c_lo + cols; c += dl.step) {
         int s[4], e[4];
 #pragma unroll
         for (int w = 0; w < 4; ++w) {
-            e[w] = (int)lds_u16(cc + 2 * (w * C + c));
-            s[w] = c ? (int)lds_u16(cc + 2 * (w * C + c) - 2) : 0;
+            e[w] = (int)lds_u16_ordered(cc + 2 * (w * C + c));
+            s[w] = c ? (int)lds_u16_ordered(cc + 2 * (w * C + c) - 2) : 0;
         }
         int done = 0;                    // tiles of the column before this bucket
 #pragma unroll
@@ -327,12 +322,12 @@ __device__ __forceinline__ void flush_rows(TablesB<NB>& T, const LayoutView& L, 
         const int b0 = 8 * n + 4 * q;
         if (b0 >= B) continue;           // absent batch rows: their sums stay zero
         const uint32_t at = smem_u32(&T.acc[0][n][r][4 * q]);
-        float4 v = lds_f32x4(at);
+        float4 v = lds_f32x4_ordered(at);
         sts_zero4(at);
 #pragma unroll
         for (int w = 1; w < NCWB; ++w) {
             const uint32_t aw = at + w * (uint32_t)sizeof(T.acc[0]);
-            const float4 o = lds_f32x4(aw);
+            const float4 o = lds_f32x4_ordered(aw);
             sts_zero4(aw);
             v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
         }
@@ -370,10 +365,10 @@ __device__ __forceinline__ void flush_cluster(TablesB<NB>& T, uint32_t stage, co
     for (int n = 0; n < NB / 8; ++n) {
         if (8 * n + 4 * q >= B) continue;
         const uint32_t at = smem_u32(&T.acc[0][n][r][4 * q]);
-        float4 v = lds_f32x4(at);
+        float4 v = lds_f32x4_ordered(at);
 #pragma unroll
         for (int w = 1; w < NCWB; ++w) {
-            const float4 o = lds_f32x4(at + w * (uint32_t)sizeof(T.acc[0]));
+            const float4 o = lds_f32x4_ordered(at + w * (uint32_t)sizeof(T.acc[0]));
             v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
         }
         if (r < rows) {
@@ -392,9 +387,9 @@ __device__ __forceinline__ void flush_cluster(TablesB<NB>& T, uint32_t stage, co
     for (int k = ct; k < mine * batch_quads(B); k += NCTB) {
         const int b4 = k / mine, row = k - b4 * mine;
         const uint32_t at = stage + (uint32_t)((row * NB + 4 * b4) * 4);
-        float4 v = lds_f32x4(at);
+        float4 v = lds_f32x4_ordered(at);
         for (int sl = 1; sl < L.S; ++sl) {
-            const float4 o = lds_f32x4(at + (uint32_t)(sl * own * NB * 4));
+            const float4 o = lds_f32x4_ordered(at + (uint32_t)(sl * own * NB * 4));
             v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
         }
         float* y = Y + (int64_t)(4 * b4) * L.N + (int64_t)rb * RB + rank * own + row;

@@ -453,7 +453,7 @@ __device__ void build_tables(ActTab<NX>& T, const LayoutView& L, const uint16_t*
                 const uint32_t a = smem_u32(T.xs) + ((c * 4 + 2 * hh + q) * XQ) * 4;
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const float4 f = lds_f32x4(a + 16 * i);
+                    const float4 f = lds_f32x4_ordered(a + 16 * i);
                     xh[16 * q + 4 * i] = f.x;
                     xh[16 * q + 4 * i + 1] = f.y;
                     xh[16 * q + 4 * i + 2] = f.z;
@@ -640,11 +640,11 @@ __device__ __forceinline__ void body1(const ActTab<NX>& T, const Task& t, uint32
 template <int NX>
 __device__ __forceinline__ void consume_unit(const ActTab<NX>& T, uint32_t sblob, uint32_t slots, int t0, int tstep,
                                              int lane) {
-    const uint32_t hw = lds_u32(sblob + offsetof(UnitHeader, ntask));     // ntask | task16 << 16
+    const uint32_t hw = lds_u32_ordered(sblob + offsetof(UnitHeader, ntask));     // ntask | task16 << 16
     const int ntask = (int)(hw & 0xFFFFu);
     const uint32_t tasks = sblob + (hw >> 16) * 16;
     for (int k = t0; k < ntask; k += tstep) {
-        const uint4 d = lds_u32x4(tasks + k * 16);
+        const uint4 d = lds_u32x4_ordered(tasks + k * 16);
         const uint32_t w = (d.x >> 26) & 3u;
         if (w == 0) body1<NX>(T, task64(sblob, d, lane), slots);
         else if (w == 1) body2<NX>(T, task32(sblob, d, lane, 16), slots);
@@ -672,9 +672,9 @@ static_assert(RB == 128, "item_pos shifts by log2(RB)");
 template <int NX, int W>
 __device__ __forceinline__ void consume_single_w(const ActTab<NX>& T, uint32_t sblob, uint32_t slots, int t0,
                                                  int tstep, int lane, int rows) {
-    const int n = (int)lds_u16(sblob + offsetof(UnitHeader, n) + 2 * W);
-    const uint32_t pay = sblob + lds_u16(sblob + offsetof(UnitHeader, pay16) + 2 * W) * 16;
-    const uint32_t sc = sblob + lds_u16(sblob + offsetof(UnitHeader, sc16) + 2 * W) * 16;
+    const int n = (int)lds_u16_ordered(sblob + offsetof(UnitHeader, n) + 2 * W);
+    const uint32_t pay = sblob + lds_u16_ordered(sblob + offsetof(UnitHeader, pay16) + 2 * W) * 16;
+    const uint32_t sc = sblob + lds_u16_ordered(sblob + offsetof(UnitHeader, sc16) + 2 * W) * 16;
     constexpr int SPAN = W == 0 ? TASK_SPAN1 : TASK_SPAN, BPI = 8 << W;
     const int ntask = (n + SPAN - 1) / SPAN;
     for (int k = t0; k < ntask; k += tstep) {
@@ -801,7 +801,7 @@ __device__ __forceinline__ void team_flush(const float* slots, const LayoutView&
         const uint32_t ra = smem_u32(slots + v * SLOT_FLOATS) + (uint32_t)r * 64;
         float sum = 0.f;
         for (int k = 0; k < chunks; ++k) {
-            const float4 a = lds_f32x4(ra + ((part * chunks + k) << 4));
+            const float4 a = lds_f32x4_ordered(ra + ((part * chunks + k) << 4));
             sum += (a.x + a.y) + (a.z + a.w);
         }
         for (int o = 1; o < lpr; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
@@ -963,7 +963,7 @@ __global__ void __launch_bounds__(G1_THREADS, 1) gemv1_kernel(LayoutView L, cons
                     const uint32_t ra = sl + (uint32_t)r * 64;
                     float4 a4[4];
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) a4[k] = lds_f32x4(ra + (((k + (lane >> 1)) & 3) << 4));
+                    for (int k = 0; k < 4; ++k) a4[k] = lds_f32x4_ordered(ra + (((k + (lane >> 1)) & 3) << 4));
                     if (rezero) {
 #pragma unroll
                         for (int k = 0; k < 4; ++k) sts_zero4(ra + (((k + (lane >> 1)) & 3) << 4));
@@ -1249,7 +1249,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) gemv_chain_kernel(const ChainIt
                             const uint32_t ra = sl + (uint32_t)r * 64;
                             float4 a[4];
 #pragma unroll
-                            for (int k = 0; k < 4; ++k) a[k] = lds_f32x4(ra + (((k + (lane >> 1)) & 3) << 4));
+                            for (int k = 0; k < 4; ++k) a[k] = lds_f32x4_ordered(ra + (((k + (lane >> 1)) & 3) << 4));
 #pragma unroll
                             for (int k = 0; k < 4; ++k) sts_zero4(ra + (((k + (lane >> 1)) & 3) << 4));
                             const float sum = (((a[0].x + a[0].y) + (a[0].z + a[0].w)) + ((a[1].x + a[1].y) + (a[1].z + a[1].w))) +
@@ -1412,7 +1412,7 @@ __global__ void __launch_bounds__(U1_THREADS, 2) gemv1_unit_kernel(LayoutView L,
     if (L.S > 1) cluster_wait();
     // row r of the unit: four lanes, a 16-byte chunk of slots each
     const int r = tid >> 2, q = tid & 3;
-    const float4 a = lds_f32x4(smem_u32(T.slots) + (uint32_t)r * 64 + (q << 4));
+    const float4 a = lds_f32x4_ordered(smem_u32(T.slots) + (uint32_t)r * 64 + (q << 4));
     float sum = (a.x + a.y) + (a.z + a.w);
     sum += __shfl_xor_sync(0xffffffffu, sum, 1);
     sum += __shfl_xor_sync(0xffffffffu, sum, 2);
