@@ -155,6 +155,29 @@ __device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
 
 __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
 
+// Reads of a product's inputs (x, X, gu), which the previous kernel on the
+// stream may still be writing when this one starts (programmatic dependent
+// launch): ordinary coherent loads that stay behind griddepcontrol.wait. (Not
+// __ldg: the read-only path is for data constant over the whole kernel, and the
+// compiler may move its loads.)
+__device__ __forceinline__ uint4 ldg_input_u32x4(const void* p) {
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint2 ldg_input_u32x2(const void* p) {
+    uint2 v;
+    asm volatile("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ float4 ldg_input_f32x4(const void* p) {
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p) : "memory");
+    return v;
+}
+
 // y += v on a global float.
 __device__ __forceinline__ void red_global(float* p, float v) {
     asm volatile("red.global.add.f32 [%0], %1;" :: "l"(p), "f"(v) : "memory");

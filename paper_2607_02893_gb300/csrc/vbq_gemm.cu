@@ -201,8 +201,8 @@ __device__ __forceinline__ void load_acts(uint32_t (&xb)[NB], const uint16_t* __
         uint4 lo = make_uint4(0u, 0u, 0u, 0u), hi = lo;
         if (8 * n + g < B) {
             const uint16_t* src = x + (int64_t)(8 * n + g) * K + 32 * (t >> 1) + 8 * (t & 1);
-            lo = __ldg(reinterpret_cast<const uint4*>(src));
-            hi = __ldg(reinterpret_cast<const uint4*>(src + 16));
+            lo = ldg_input_u32x4(src);
+            hi = ldg_input_u32x4(src + 16);
         }
         const uint32_t a[4] = {lo.x, lo.y, lo.z, lo.w}, b[4] = {hi.x, hi.y, hi.z, hi.w};
 #pragma unroll

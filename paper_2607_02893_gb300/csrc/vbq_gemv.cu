@@ -377,14 +377,14 @@ __device__ void build_tables(ActTab<NX>& T, const LayoutView& L, const uint16_t*
             if constexpr (MODE == MODE_SWIGLU_IN) {
                 // SwiGLU input: activation k is silu(gu[2k]) * gu[2k + 1]
                 const float4* src = reinterpret_cast<const float4*>(gu + 2 * ((int64_t)s * L.C * GROUP + c * GROUP + jj));
-                const float4 a = __ldg(src), b = __ldg(src + 1);
+                const float4 a = ldg_input_f32x4(src), b = ldg_input_f32x4(src + 1);
                 x0 = swiglu_f32(a.x, a.y);
                 x1 = swiglu_f32(a.z, a.w);
                 x2 = swiglu_f32(b.x, b.y);
                 x3 = swiglu_f32(b.z, b.w);
             } else {
                 const uint16_t* xg = x + (int64_t)v * L.K + (int64_t)s * L.C * GROUP;
-                const uint2 four = __ldg(reinterpret_cast<const uint2*>(xg + c * GROUP + jj));
+                const uint2 four = ldg_input_u32x2(xg + c * GROUP + jj);
                 x0 = __uint_as_float(four.x << 16);
                 x1 = __uint_as_float(four.x & 0xFFFF0000u);
                 x2 = __uint_as_float(four.y << 16);
@@ -429,7 +429,7 @@ __device__ void build_tables(ActTab<NX>& T, const LayoutView& L, const uint16_t*
             float xh[32];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const uint4 w = __ldg(src + q);
+                const uint4 w = ldg_input_u32x4(src + q);
                 const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
