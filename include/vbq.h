@@ -30,10 +30,11 @@
  *   - Device arrays must be 16-byte aligned (VBQ_ERR_ALIGN otherwise).
  *   - The library keeps per-device state for the life of the process (each
  *     kernel's shared-memory limit, set once per device; the device address
- *     of vbq_gemv_static's array). A device reset (cudaDeviceReset), or
- *     anything else that destroys and recreates the device's primary
- *     context, invalidates that state: do not call the library on that
- *     device afterwards in the same process.
+ *     of vbq_gemv_static's array; a 4 KB page of pinned host memory through
+ *     which vbq_quantize and vbq_pack report errors). A device reset
+ *     (cudaDeviceReset), or anything else that destroys and recreates the
+ *     device's primary context, invalidates that state: do not call the
+ *     library on that device afterwards in the same process.
  *   - Activations (BF16) must be finite with magnitude below 2^64; larger
  *     values may overflow inside the kernels' scaled arithmetic.
  */

@@ -5,10 +5,10 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
-#include <mutex>
 #include <vector>
 
 #include "../../include/vbq.h"
+#include "vbq_error_words.h"
 #include "vbq_kernels.h"
 
 struct vbq_layout {
@@ -56,74 +56,6 @@ struct TempBuffers {
         return e;
     }
 };
-
-// Two error words of one call, in pinned host memory that every device can
-// write: a validating kernel stores to them only on an error, and the host
-// reads them once it has synchronised, without a copy or an allocation per
-// call. The words come from one page shared by all threads (64 calls at a
-// time, one 64-byte line each, given back when the call ends); a call beyond
-// those allocates its own.
-class ErrorWords {
-public:
-    // The words may be another call's next: a kernel of this one that has not
-    // been synchronised with (an error on the way out) is waited for first.
-    ~ErrorWords() {
-        if (armed_) cudaStreamSynchronize(stream_);
-        if (slot_ >= 0) {
-            std::lock_guard<std::mutex> lock(mu_);
-            used_ &= ~(1ull << slot_);
-        } else if (w_) {
-            cudaFreeHost(w_);
-        }
-    }
-    cudaError_t get(cudaStream_t stream) {
-        stream_ = stream;
-        {
-            std::lock_guard<std::mutex> lock(mu_);
-            if (!page_) {
-                const cudaError_t e = host_words(&page_, 4096);
-                if (e != cudaSuccess) return e;
-            }
-            for (int i = 0; i < 64 && slot_ < 0; ++i)
-                if (!(used_ >> i & 1)) slot_ = i;
-            if (slot_ >= 0) {
-                used_ |= 1ull << slot_;
-                w_ = page_ + 16 * slot_;
-            }
-        }
-        if (!w_) {
-            const cudaError_t e = host_words(&w_, 64);
-            if (e != cudaSuccess) return e;
-        }
-        w_[0] = w_[1] = 0;
-        return cudaSuccess;
-    }
-    uint32_t* arm(int i) {                  // for a kernel about to be launched on the stream
-        armed_ = true;
-        return w_ + i;
-    }
-    cudaError_t settle() {                  // wait for the stream; the words can be read
-        const cudaError_t e = cudaStreamSynchronize(stream_);
-        armed_ = false;
-        return e;
-    }
-    bool set(int i) const { return static_cast<volatile uint32_t*>(w_)[i] != 0; }
-
-private:
-    static cudaError_t host_words(uint32_t** p, size_t bytes) {
-        return cudaHostAlloc(reinterpret_cast<void**>(p), bytes, cudaHostAllocPortable | cudaHostAllocMapped);
-    }
-    static std::mutex mu_;
-    static uint32_t* page_;
-    static uint64_t used_;
-    uint32_t* w_ = nullptr;
-    int slot_ = -1;
-    cudaStream_t stream_ = nullptr;
-    bool armed_ = false;
-};
-std::mutex ErrorWords::mu_;
-uint32_t* ErrorWords::page_ = nullptr;
-uint64_t ErrorWords::used_ = 0;
 
 #define VBQ_CUDA(call)                                                                     \
     do {                                                                                   \
@@ -197,7 +129,7 @@ vbq_status_t vbq_pack(const uint8_t* codes, const uint8_t* bitwidths, const uint
     const int64_t G = K / vbq::GROUP;
     const size_t ncodes = (size_t)N * (size_t)K, ngroups = (size_t)N * (size_t)G;
     TempBuffers tmp;
-    ErrorWords err;
+    vbq::ErrorWords err;
     VBQ_CUDA(err.get(s));
 
     const uint8_t* d_codes = codes;
@@ -384,7 +316,7 @@ vbq_status_t vbq_quantize(const float* w, const uint8_t* bitwidths, int64_t N, i
     if (!aligned16(w) || !aligned16(bitwidths) || !aligned16(codes_out) || !aligned16(scales_out))
         return fail(VBQ_ERR_ALIGN, "device arrays must be 16-byte aligned");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    ErrorWords err;
+    vbq::ErrorWords err;
     VBQ_CUDA(err.get(s));
     VBQ_CUDA(vbq::launch_quant_validate(w, bitwidths, N, K, err.arm(0), s));
     VBQ_CUDA(err.settle());
