@@ -126,6 +126,8 @@ class Layout:
 
     def __init__(self, handle: int, n: int, k: int):
         self.handle = handle
+        # made once: a pointer in any ctypes call (a plain integer is one only where argtypes say so)
+        self._param = ctypes.c_void_p(handle)
         self.N = n
         self.K = k
 
@@ -144,7 +146,7 @@ class Layout:
     def _as_parameter_(self):
         if not self.handle:
             raise ValueError("layout already freed")
-        return self.handle
+        return self._param
 
 
 def vbq_quantize(w, bitwidths, codes_out=None, scales_out=None, stream=None):
