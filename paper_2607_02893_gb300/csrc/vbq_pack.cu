@@ -332,17 +332,18 @@ __device__ __forceinline__ uint32_t item_codes4(const uint8_t* src, int w, int l
     return w == 0 ? lo : lo | (spread_bits((p[2 + (l >> 3)] >> sh) & 0xFu) << 1);
 }
 
-// One block per unit: the blob into shared memory, the item of every (row,
-// column) by one pass over the row bytes, then the groups in row order, two
-// at a time per warp (16 lanes, four codes each), so that a warp writes whole
-// 256-byte groups of floats. Bound: HBM, by the outputs. (One thread per item
-// wrote 256 bytes on its own: 322 us for all outputs of 14336 x 4096, now
-// 54 us.)
+// gridDim.y blocks per unit: the blob into shared memory, the item of every
+// (row, column) by one pass over the row bytes, then the groups in row order
+// (each block its share, `per` at a time per warp), two at once per warp (16
+// lanes, four codes each), so that a warp writes whole 256-byte groups of floats.
+// Bound: HBM, by the outputs. (One thread per item wrote 256 bytes on its own:
+// 322 us for all outputs of 14336 x 4096, now 54 us.) Small layouts are bound by
+// the latency of a warp's groups one after another: see launch_dequant.
 constexpr int DQ_THREADS = 256;
 
 __global__ void __launch_bounds__(DQ_THREADS) dequant_kernel(LayoutView L, uint8_t* codes_out,
                                                              uint8_t* widths_out, uint16_t* scales_out,
-                                                             float* w_out) {
+                                                             float* w_out, int per) {
     __shared__ __align__(16) uint8_t blob[MAX_BLOB_BYTES];
     __shared__ uint16_t item_of[MAX_C * RB];            // width index << 12 | item
     const int u = blockIdx.x, rb = unit_rb(L, u), s = unit_slab(L, u);
@@ -365,7 +366,8 @@ __global__ void __launch_bounds__(DQ_THREADS) dequant_kernel(LayoutView L, uint8
     __syncthreads();
     const int total = rows * cols;
     const int64_t g00 = (int64_t)rb * RB * L.G + (int64_t)s * L.C;
-    for (int base = 32 * warp; base < total; base += DQ_THREADS) {
+    const int pass = per * (DQ_THREADS / 32);           // groups per block and pass
+    for (int base = per * warp + pass * blockIdx.y; base < total; base += pass * gridDim.y) {
         // lane's group, in row order
         const int p = base + lane, pv = min(p, total - 1);
         const int r = pv / cols, c = pv - r * cols;
@@ -373,14 +375,15 @@ __global__ void __launch_bounds__(DQ_THREADS) dequant_kernel(LayoutView L, uint8
         const uint16_t sbits = reinterpret_cast<const uint16_t*>(blob + h.sc16[w] * 16)[it];
         const uint32_t pay = h.pay16[w] * 16u + it * (8u << w);
         const int64_t g = g00 + (int64_t)r * L.G + c;
-        if (p < total) {
+        if (lane < per && p < total) {
             if (widths_out) widths_out[g] = (uint8_t)(1u << w);
             if (scales_out) scales_out[g] = sbits;
         }
         if (!codes_out && !w_out) continue;
         const float sf = __half2float(__ushort_as_half(sbits));
-        const int nb = min(32, total - base);
+        const int nb = min(per, total - base);
         const int l = lane & 15;
+#pragma unroll 4
         for (int k = 0; k < nb; k += 2) {
             const int src = k + (lane >> 4);
             const uint32_t pk = __shfl_sync(0xffffffffu, pay | (w << 16), src);
@@ -425,7 +428,22 @@ cudaError_t launch_scatter(const uint8_t* codes, const uint8_t* widths, const ui
 
 cudaError_t launch_dequant(const LayoutView& L, uint8_t* codes_out, uint8_t* widths_out,
                            uint16_t* scales_out, float* w_out, cudaStream_t s) {
-    dequant_kernel<<<L.units, DQ_THREADS, 0, s>>>(L, codes_out, widths_out, scales_out, w_out);
+    int sms = 0;
+    const int err = device_sms(&sms);
+    if (err != 0) return (cudaError_t)err;
+    // Codes and weights of a layout with few units are bound by latency: a warp's
+    // 32 groups take about 2.5 us, two at a time, and a unit's several passes
+    // follow one another. So while blocks are fewer than two per SM a unit's
+    // passes go to several blocks, of 16 groups a warp where those all fit (us
+    // for the codes: 256 x 2048 7.7 -> 4.0, 768 x 768 4.8 -> 3.6; 2048 x 2048, of
+    // 32 groups, 7.8 -> 5.7; 4096 x 4096 24.6 -> 15.4).
+    int per = 32, parts = 1;
+    if (codes_out || w_out) {
+        const int64_t fit = 2 * (int64_t)sms;
+        if (L.units * (int64_t)(RB * L.C / 128) <= fit) per = 16;
+        while (L.units * (int64_t)parts < fit && per * (DQ_THREADS / 32) * parts < RB * L.C) parts *= 2;
+    }
+    dequant_kernel<<<dim3(L.units, parts), DQ_THREADS, 0, s>>>(L, codes_out, widths_out, scales_out, w_out, per);
     return cudaGetLastError();
 }
 
