@@ -459,10 +459,15 @@ vbq_status_t vbq_chain_create(const vbq_layout* const* layouts, const uint16_t* 
             it.wait_from = it.wait_hi = i;
         }
         it.rot = (int)(units_before % sms);
+        it.awaited = 0;
         units_before += it.L.units;
         seen_l[i] = layouts[i];
         seen_y[i] = ys[i];
     }
+    // products are waited for in ranges that begin where the last one ended (or repeat it)
+    for (int i = 0, marked = 0; i < count; ++i)
+        for (marked = std::max(marked, items[(size_t)i].wait_from); marked < items[(size_t)i].wait_hi; ++marked)
+            items[(size_t)marked].awaited = 1;
     std::sort(seen_l.begin(), seen_l.end());
     std::sort(seen_y.begin(), seen_y.end());
     if (std::adjacent_find(seen_l.begin(), seen_l.end()) != seen_l.end())

@@ -166,6 +166,7 @@ struct ChainItem {
     int wait_from;
     int wait_hi;
     int rot;
+    int awaited;                // some later product waits for this one
 };
 
 __host__ __device__ inline int width_of(int w) { return 1 << w; }
