@@ -142,10 +142,11 @@ vbq_status_t vbq_soft_quant(const float* w, const float* logits, const float* gu
  *   stream       stream for the device work.
  *   out          receives the new layout on VBQ_OK.
  *
- * Validates shape, widths and code ranges (VBQ_ERR_SHAPE / _WIDTH /
- * _CODE_RANGE) before building anything. The layout owns its device memory
- * until vbq_free. This call synchronises `stream` (it reads back counts to
- * size the allocation) and may allocate temporary device memory.
+ * Validates shape and widths (VBQ_ERR_SHAPE / _WIDTH) before building
+ * anything, and code ranges (_CODE_RANGE) while building: on any error nothing
+ * stays allocated and *out is NULL. The layout owns its device memory until
+ * vbq_free. This call synchronises `stream` (it reads back counts to size the
+ * allocation) and may allocate temporary device memory.
  */
 vbq_status_t vbq_pack(const uint8_t* codes, const uint8_t* bitwidths,
                       const uint16_t* scales_fp16, int64_t N, int64_t K,
@@ -184,11 +185,10 @@ vbq_status_t vbq_dequant(const vbq_layout* layout, uint8_t* codes_out,
  *   x  device, K BF16 bit patterns.
  *   y  device, N floats; overwritten.
  * Per output, |y - y_exact| stays within 2e-3 * sum_k |w_nk x_k| + 1e-5.
- * Groups of one row block are summed in a varying order, so repeated calls can
- * differ in the last bits. When a row spans several slabs of the layout, the
- * call uses a split-K workspace
- * owned by the layout: calls that share a layout must not overlap on the GPU
- * (issue them on one stream, or order them with events). The kernel is
+ * When a row spans several slabs of the layout, their sums may be added in a
+ * varying order, so repeated calls can differ in the last bits, and the call may
+ * use a split-K workspace owned by the layout: calls that share a layout must
+ * not overlap on the GPU (issue them on one stream, or order them with events). The kernel is
  * launched with programmatic dependent launch: it may start loading weights
  * before the previous kernel on the stream has finished, and reads x only
  * after it has.
@@ -205,10 +205,10 @@ vbq_status_t vbq_gemv(const vbq_layout* layout, const uint16_t* x, float* y,
  * can differ in the last bits between calls). For B = 2..4 the library picks,
  * from the layout's group count per width, the cheaper of two paths: the
  * batch-1 table kernel, two rows per launch (both rows share every lookup
- * address and decoded code) and a single row for an odd count, each row
- * computed as vbq_gemv computes it; or the tensor cores (chosen for layouts
- * heavy in 4- and 8-bit groups, and for most mixes from three
- * rows on). For B >= 5 the product runs on the tensor cores: activations as
+ * address and decoded code) and a single row for an odd count, each group's
+ * sum computed as vbq_gemv computes it (a row's slabs may be added in another
+ * order); or the tensor cores (chosen for layouts heavy in 4- and 8-bit groups,
+ * and for most mixes from three rows on). For B >= 5 the product runs on the tensor cores: activations as
  * they are (BF16), weights as exact levels, fp32 accumulation. Y needs no
  * zeroing; the same split-K workspace and ordering rules as vbq_gemv apply
  * (calls sharing a layout must not overlap on the GPU), and the kernels are

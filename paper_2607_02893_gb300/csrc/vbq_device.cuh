@@ -190,9 +190,6 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
     asm volatile("prefetch.global.L2 [%0];" :: "l"(p));
 }
 
-// Order this thread's earlier writes (and those it has observed) before its
-// later ones, GPU-wide: the release half of __threadfence, without waiting for
-// sequential consistency.
 // Release store / acquire load at GPU scope: the split-K zeroed-row flags.
 // A warp's zero stores, ordered before lane 0 by the warp barrier, are visible
 // to whoever acquires the flag; the acquiring lanes order the warp's later

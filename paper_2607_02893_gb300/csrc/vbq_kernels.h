@@ -59,9 +59,11 @@ inline bool unit_plan_fits(int64_t C, int64_t S, int64_t units, int64_t groups, 
 // fused products (4096x4096, 262,144 groups, between 6144x4096 and
 // 28672x4096) take 36.9 us with 4096x4096 on the persistent kernel and 39.0 on
 // this one, and its 1024x4096 products among 4096x4096 ones cost the unfused
-// layer 0.5 us; a ~1B layer, all but the head below the line, takes 22.8
-// instead of 26.1. So a matrix stays off it when it, or a square matrix on its
-// input (what its neighbours are like), has 200,000 groups or more.
+// layer 0.5 us; a ~1B layer, of which only the down projection (2048x5632) stays
+// off it, takes 22.8 instead of 26.1. So a matrix stays off it when it, or a
+// square matrix on its input, has 200,000 groups or more: K stands for what the
+// neighbours are like, which a call cannot see (a single 1024x4096 product, or
+// one among small ones, is kept off it too).
 inline bool unit_neighbours(int64_t G) { return GROUP * G * G < UNIT_MAX_GROUPS; }
 inline bool runs_unit_per_block(const LayoutView& L, int sms) {
     return unit_neighbours(L.G) && unit_plan_fits(L.C, L.S, L.units, L.N * L.G, sms);

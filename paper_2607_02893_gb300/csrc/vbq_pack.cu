@@ -127,11 +127,12 @@ __global__ void __launch_bounds__(RB) count_kernel(const uint8_t* __restrict__ w
 // decreasing cost, each to the least-loaded of 16 bins that still has a
 // position (bin b holds positions b, b + 16, ...; the first nt % 16 bins one
 // more than the rest, so the positions are exactly 0 .. nt - 1; bins b and
-// b + 8 together are a warp's share when tw = 8). The costs are the batch-1
-// kernel's time per group and width (measured: 5.33, 7.02, 9.98, 14.0 units for
-// 1, 2, 4, 8 bits) times a task's items: a task
-// costs its full span even when shorter, since idle lanes repeat its first
-// item. The order does not change any result: every group has its own slot.
+// b + 8 together are a warp's share when tw = 8). The costs are a time per group
+// and width (5.33, 7.02, 9.98, 14.0 units for 1, 2, 4, 8 bits, measured on an
+// earlier form of the batch-1 kernel) times a task's items: a task costs its full
+// span even when shorter, since idle lanes repeat its first item. The kernel's
+// costs since (4.09, 5.86, 8.78, 13.1, vbq_plan.cu) give the same times: ~9B layer
+// 45.7 us with either, head 36.8, ~131M step 196.4. The order does not change any result: every group has its own slot.
 // One warp: lane b < 16 is bin b, and the least-loaded bin is one warp
 // reduction (a single thread scanning the bins took about 50 us a unit).
 // in: the tasks of widths 8, 4, 2, 1 bits, of which width w has n[w] from off[w].

@@ -12,7 +12,12 @@ namespace vbq {
 // on it, and four rows on the tensor cores. The tensor cores take items in
 // tiles of 16 from each (column, width) bucket of a unit, so a bucket leaves
 // about 6 item slots of its last tile idle (16384 x 16384 of the main mix: 50
-// us measured at 4 rows, 55 us modelled). So two rows of a 1- or 2-bit heavy
+// us measured at 4 rows, 55 us modelled). They are charged also where a
+// single-width matrix fills its tiles, which keeps two rows of an all-2-bit one
+// on the tables: the faster side on small matrices (4096 x 4096 5.9 us, 7.2 on
+// the tensor cores), the slower one on large ones (14336 x 4096 12.1, 11.2).
+// Narrow units are charged like wide ones, though both sides cost more on them.
+// So two rows of a 1- or 2-bit heavy
 // matrix stay on the tables (main mix 43 us) and three or four go to the
 // tensor cores (64 and 83 us on the tables).
 constexpr double COST_ONE[4] = {4.09, 5.86, 8.78, 13.1};
