@@ -226,10 +226,10 @@ __device__ __forceinline__ void run_tiles(const DecodeConsts& K, const uint32_t 
     sc += k0 * 32;
     rw += k0 * 16;
     for (int left = n - 16 * k0; left > 0; left -= 16 * kstep) {
+        const uint32_t sa = lds_u16_ordered(sc), sb = lds_u16_ordered(sc + 16), ra = lds_u8(rw), rb = lds_u8(rw + 8);
         uint32_t la[8], lb[8];
         levels<W>(K, pay, sh, la);
         levels<W>(K, pay + 8 * BPI, sh, lb);
-        const uint32_t sa = lds_u16(sc), sb = lds_u16(sc + 16), ra = lds_u8(rw), rb = lds_u8(rw + 8);
         float d[NB / 8][4];
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
@@ -274,14 +274,16 @@ __device__ __forceinline__ Deal deal_columns(int cols, int cw) {
 }
 
 // One warp's share of columns [c_lo, c_lo + cols) of a unit (blob at sblob,
-// activations of its slab at x); xb holds the first column's activations.
+// activations of its slab at x); xb holds the first column's activations. A
+// bucket's offsets are read from the header as it begins: held over the unit
+// they took 12 registers of the tile loops (16384^2 all 8 bits at 4 rows 89.2 us,
+// 87.0; 14336 x 4096 main at 16 rows 17.8, 17.0).
 template <int NB>
 __device__ __forceinline__ void consume_unit_b(const DecodeConsts& K, uint32_t sblob, int C, int c_lo, int cols, const Deal& dl,
                                                uint32_t (&xb)[NB], const uint16_t* __restrict__ x, int64_t Kx, int B,
                                                uint32_t acc, int lane) {
     const int g = lane >> 2, t = lane & 3, sh = 8 * (t & 1);
-    const uint4 h0 = lds_u32x4_ordered(sblob), h1 = lds_u32x4_ordered(sblob + 16), h2 = lds_u32x4_ordered(sblob + 32);
-    const uint32_t cc = sblob + (h2.x & 0xFFFF) * 16;
+    const uint32_t cc = sblob + lds_u16_ordered(sblob + offsetof(UnitHeader, cc16)) * 16;
     const uint32_t my = acc + 8u * t;
     for (int c = c_lo + dl.c0; c < c_lo + cols; c += dl.step) {
         int s[4], e[4];
@@ -294,9 +296,9 @@ __device__ __forceinline__ void consume_unit_b(const DecodeConsts& K, uint32_t s
 #pragma unroll
         for (int w = 0; w < 4; ++w) {
             const int n = e[w] - s[w], first = s[w] + g;
-            const uint32_t p16 = w == 0 ? h0.z & 0xFFFF : w == 1 ? h0.z >> 16 : w == 2 ? h0.w & 0xFFFF : h0.w >> 16;
-            const uint32_t s16 = w == 0 ? h1.x & 0xFFFF : w == 1 ? h1.x >> 16 : w == 2 ? h1.y & 0xFFFF : h1.y >> 16;
-            const uint32_t r16 = w == 0 ? h1.z & 0xFFFF : w == 1 ? h1.z >> 16 : w == 2 ? h1.w & 0xFFFF : h1.w >> 16;
+            const uint32_t p16 = lds_u16_ordered(sblob + offsetof(UnitHeader, pay16) + 2 * w);
+            const uint32_t s16 = lds_u16_ordered(sblob + offsetof(UnitHeader, sc16) + 2 * w);
+            const uint32_t r16 = lds_u16_ordered(sblob + offsetof(UnitHeader, row16) + 2 * w);
             const uint32_t pay = sblob + p16 * 16 + first * (8 << w), sc = sblob + s16 * 16 + first * 2, rw = sblob + r16 * 16 + first;
             const int k0 = (dl.sub - done) & (dl.parts - 1);
             if (w == 0) run_tiles<NB, 0>(K, xb, pay + lane_offset<0>(t), sc, rw, n, k0, dl.parts, my, g, sh);
@@ -400,7 +402,12 @@ __device__ __forceinline__ void flush_cluster(TablesB<NB>& T, uint32_t stage, co
     }
 }
 
-template <int NB, bool CL>
+// How a launch's units go to its blocks, each form an instantiation of its own:
+// evenly, with left-over units cut (see Shares), or a row block's slabs as a
+// cluster.
+enum Split : int { SPLIT_EVEN, SPLIT_CUT, SPLIT_CLUSTER };
+
+template <int NB, int SPLIT>
 __global__ void __launch_bounds__(GB_THREADS, GB_BLOCKS) gemmb_kernel(LayoutView L, const uint16_t* __restrict__ X,
                                                                       float* __restrict__ Y, int B, Shares sh) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -409,6 +416,7 @@ __global__ void __launch_bounds__(GB_THREADS, GB_BLOCKS) gemmb_kernel(LayoutView
     const uint32_t stage = smem_u32(base);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int P = gridDim.x, p = blockIdx.x;
+    constexpr bool CL = SPLIT == SPLIT_CLUSTER, CUT = SPLIT == SPLIT_CUT;
     // the block's places in the deal: begin, begin + 1, ..., and perhaps a part of another
     int begin, whole, part_at = -1, part = 0;
     if (CL) {                            // block rb * S + s: unit (rb, s)
@@ -416,13 +424,15 @@ __global__ void __launch_bounds__(GB_THREADS, GB_BLOCKS) gemmb_kernel(LayoutView
         begin = (p - rb * L.S) * L.nrb + rb;
         whole = 1;
     } else {
-        const BlockShare b = block_share(L.units, sh, P, p);
+        const BlockShare b = block_share(L.units, CUT ? sh : Shares{0, 0, 1, 0}, P, p);
         begin = b.begin;
         whole = b.whole;
-        part_at = b.part_at;
-        part = b.part;
+        if (CUT) {
+            part_at = b.part_at;
+            part = b.part;
+        }
     }
-    const int n_units = whole + (part_at >= 0), rot = CL ? 0 : sh.rot;
+    const int n_units = whole + (part_at >= 0), rot = CUT ? sh.rot : 0;
     auto place = [&](int j) { return j < whole ? begin + j : part_at; };
     // the block that zeroes Y's rows of place j's row block (under split-K; slab 0 is dealt in order)
     auto owns_zeroing = [&](int j) { return place(j) < L.nrb && (j < whole || part == 0); };
@@ -523,14 +533,22 @@ __global__ void __launch_bounds__(GB_THREADS, GB_BLOCKS) gemmb_kernel(LayoutView
         if (L.S > 1 && lane == 0) red_release_cta_shared_add(smem_u32(&T.sk_ok), dead ? 0x10000u : 1u);
         int issued = 1;
         for (int j = 0; j + 1 < n_units && !dead; ++j) {
+            // A refill's latency is on the block's path (one stage). With narrow units,
+            // of few groups for their bytes, its offsets are read before the stage
+            // is free (16384^2 all 4 bits at 4 rows 53.3 us, 55.7 otherwise); with
+            // 16-column units that loses 1% (8192^2 main 15.1, 15.3).
+            const int d = place(j + 1), sl = d / L.nrb, u = sl * L.nrb + dealt_row_block(d, sl, L.nrb, rot);
+            const bool early = L.C < MAX_C;
+            uint32_t o0 = 0, o1 = 0;
+            if (early) { o0 = L.blob_off[u]; o1 = L.blob_off[u + 1]; }
             if (!warp_wait(empty, (uint32_t)j & 1u, abort_addr, 128)) {
                 dead = true;
                 if (lane == 0) raise_abort(&T.abort);
                 break;
             }
             if (lane == 0) {
-                const int d = place(j + 1), sl = d / L.nrb;
-                issue_unit(L, sl * L.nrb + dealt_row_block(d, sl, L.nrb, rot), stage, full);
+                if (early) bulk_load(stage, L.blobs + (int64_t)o0 * 16, (o1 - o0) * 16, full);
+                else issue_unit(L, u, stage, full);
             }
             ++issued;
         }
@@ -556,7 +574,7 @@ __global__ void __launch_bounds__(GB_THREADS, GB_BLOCKS) gemmb_kernel(LayoutView
         for (int j = 0; j < n_units; ++j) {
             const int d = place(j), sj = d / L.nrb, rbj = dealt_row_block(d, sj, L.nrb, rot);
             int cols = min(L.C, L.G - sj * L.C), c_lo = 0;
-            if (!CL && j >= whole) {     // a part: its share of the columns
+            if (CUT && j >= whole) {     // a part: its share of the columns
                 c_lo = cols * part / sh.parts;
                 cols = cols * (part + 1) / sh.parts - c_lo;
             }
@@ -597,7 +615,7 @@ __global__ void __launch_bounds__(GB_THREADS, GB_BLOCKS) gemmb_kernel(LayoutView
     }
 }
 
-template <int NB, bool CL>
+template <int NB, int SPLIT>
 cudaError_t launch_gemmb(const LayoutView& L, const uint16_t* X, float* Y, int B, cudaStream_t s, int grid, Shares sh) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
@@ -612,8 +630,8 @@ cudaError_t launch_gemmb(const LayoutView& L, const uint16_t* X, float* Y, int B
     attr[1].val.clusterDim.y = 1;
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = CL ? 2 : 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, gemmb_kernel<NB, CL>, L, X, Y, B, sh);
+    cfg.numAttrs = SPLIT == SPLIT_CLUSTER ? 2 : 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, gemmb_kernel<NB, SPLIT>, L, X, Y, B, sh);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
@@ -635,20 +653,24 @@ cudaError_t launch_gemmb(const LayoutView& L, const uint16_t* X, float* Y, int B
 // 15.1 -> 12.6 and 20.9 -> 17.6.
 template <int NB>
 cudaError_t launch_gemm(const LayoutView& L, const uint16_t* X, float* Y, int B, cudaStream_t s) {
-    static LaunchPrep prep, prep_cl;
+    static LaunchPrep prep, prep_cut, prep_cl;
     int sms = 0;
-    cudaError_t e = prep.get(gemmb_kernel<NB, false>, gemmb_smem<NB>(), &sms);
+    cudaError_t e = prep.get(gemmb_kernel<NB, SPLIT_EVEN>, gemmb_smem<NB>(), &sms);
     if (e != cudaSuccess) return e;
     constexpr int64_t SMALL = 50000;
     const bool pays = NB == 16 ? L.S <= MAX_CLUSTER
                                : B > 4 && L.S <= 8 && L.N * L.G < SMALL && GROUP * (int64_t)L.G * L.G < SMALL;
     if (pays && L.S > 1 && L.C <= 8 && 4 * (int64_t)L.units <= (L.S <= 8 ? 7 : 5) * (int64_t)sms) {
-        if ((e = prep_cl.get(gemmb_kernel<NB, true>, gemmb_smem<NB>(), &sms, true)) != cudaSuccess) return e;
-        return launch_gemmb<NB, true>(L, X, Y, B, s, L.units, Shares{0, 0, 1, 0});
+        if ((e = prep_cl.get(gemmb_kernel<NB, SPLIT_CLUSTER>, gemmb_smem<NB>(), &sms, true)) != cudaSuccess) return e;
+        return launch_gemmb<NB, SPLIT_CLUSTER>(L, X, Y, B, s, L.units, Shares{0, 0, 1, 0});
     }
     const int blocks = GB_BLOCKS * sms;
     const Shares sh = plan_shares(L.units, L.nrb, L.S, L.C == 2 * NCWB, blocks);
-    return launch_gemmb<NB, false>(L, X, Y, B, s, grid_blocks(L.units, sh, blocks), sh);
+    if (sh.parts > 1) {
+        if ((e = prep_cut.get(gemmb_kernel<NB, SPLIT_CUT>, gemmb_smem<NB>(), &sms)) != cudaSuccess) return e;
+        return launch_gemmb<NB, SPLIT_CUT>(L, X, Y, B, s, grid_blocks(L.units, sh, blocks), sh);
+    }
+    return launch_gemmb<NB, SPLIT_EVEN>(L, X, Y, B, s, grid_blocks(L.units, sh, blocks), sh);
 }
 
 }  // namespace
