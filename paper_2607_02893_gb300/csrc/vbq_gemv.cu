@@ -55,6 +55,8 @@
 // block's slab count reads the finished rows back); MODE_SWIGLU_IN, on the
 // down projection, builds its activation tables from h_k = silu(gu[2k]) *
 // gu[2k + 1] of the gate-up product's fp32 output, so h never reaches memory.
+#include <type_traits>
+
 #include <cstddef>
 #include <mutex>
 
@@ -653,6 +655,77 @@ __device__ __forceinline__ void consume_unit(const ActTab<NX>& T, uint32_t sblob
     }
 }
 
+// A wide view of a layout for two activation vectors: up to MAX_C columns of
+// neighbouring slabs as one slab, a row block's blobs of them side by side in
+// one stage (blob_stride apart). Small matrices are packed in slabs narrower
+// than gemv1_kernel<2> works best on (it does not run one unit per block): every
+// unit costs it a wait, a flush of both vectors' rows and additions into y. The
+// slab width is the one that gives at least half as many units as SMs, as larger
+// matrices are packed, if its blobs fit a stage.
+// Four matrices in turn, in a graph, per call of two rows, narrow units -> wide
+// view (us): 5632x2048 main 6.1 -> 5.7, all 1 bit 6.6 -> 4.8; 6016x1600 6.4 ->
+// 5.3; 8192x1536 6.4 -> 5.5. (For one vector and for chains the second blob's cost is not made up:
+// 14336x4096 in a chain, with the loop over one blob, 8.6 -> 9.4.)
+struct WideView {
+    LayoutView L;                           // slabs, units and columns as the kernel takes them
+    int sub = 1, slabs = 1, cols = 0;       // layout slabs per slab, of them in all, their columns
+    uint32_t blob_stride = 0;
+};
+WideView wide_view(const LayoutView& L, int sms) {
+    WideView V;
+    V.L = L;
+    V.slabs = L.S;
+    V.cols = L.C;
+    V.blob_stride = (uint32_t)L.max_blob16 * 16u;
+    int c = MAX_C;
+    while (c > 1 && (c > L.G || 2 * (int64_t)L.nrb * ((L.G + c - 1) / c) < sms)) c /= 2;
+    int sub = c / L.C;
+    while (sub > 1 && sub * V.blob_stride > MAX_BLOB_BYTES) sub /= 2;
+    if (sub <= 1) return V;
+    V.sub = sub;
+    V.L.C = L.C * sub;
+    V.L.S = (L.G + V.L.C - 1) / V.L.C;
+    V.L.units = V.L.nrb * V.L.S;
+    return V;
+}
+__device__ __forceinline__ const LayoutView& layout_of(const LayoutView& L) { return L; }
+__device__ __forceinline__ const LayoutView& layout_of(const WideView& V) { return V.L; }
+__device__ __forceinline__ int wide_parts(const WideView& V, int slab) { return min(V.sub, V.slabs - slab * V.sub); }
+__device__ __forceinline__ void issue_wide(const WideView& V, int u, uint32_t dst, uint32_t bar) {
+    const int s = u / V.L.nrb, rb = u - s * V.L.nrb, n = wide_parts(V, s);
+    const uint32_t* off = V.L.blob_off + s * V.sub * V.L.nrb + rb;
+    uint32_t bytes = 0;
+    for (int k = 0; k < n; ++k) bytes += (off[k * V.L.nrb + 1] - off[k * V.L.nrb]) * 16u;
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(bar), "r"(bytes) : "memory");
+    for (int k = 0; k < n; ++k) {
+        const uint32_t o0 = off[k * V.L.nrb], o1 = off[k * V.L.nrb + 1];
+        bulk_copy(dst + k * V.blob_stride, V.L.blobs + (int64_t)o0 * 16, (o1 - o0) * 16, bar);
+    }
+}
+// consume_unit over the unit's blobs, whose columns follow one another in the
+// tables and slots; the deal of tasks to warps runs on from blob to blob.
+template <int NX>
+__device__ __forceinline__ void consume_wide(const ActTab<NX>& T, const WideView& V, int slab, uint32_t stage, uint32_t slots,
+                                             int t0, int tstep, int lane) {
+    const int n = wide_parts(V, slab);
+    for (int b = 0; b < n; ++b) {
+        const uint32_t sblob = stage + b * V.blob_stride;
+        const uint32_t hw = lds_u32_ordered(sblob + offsetof(UnitHeader, ntask));
+        const int ntask = (int)(hw & 0xFFFFu);
+        const uint32_t tasks = sblob + (hw >> 16) * 16;
+        for (int k = t0; k < ntask; k += tstep) {
+            uint4 d = lds_u32x4_ordered(tasks + k * 16);
+            d.x += (uint32_t)(b * V.cols) << 16;            // the task's first column
+            const uint32_t w = (d.x >> 26) & 3u;
+            if (w == 0) body1<NX>(T, task64(sblob, d, lane), slots);
+            else if (w == 1) body2<NX>(T, task32(sblob, d, lane, 16), slots);
+            else if (w == 2) body4<NX>(T, task32(sblob, d, lane, 32), slots, lane);
+            else body8<NX>(T, task32(sblob, d, lane, 64), slots, lane);
+        }
+        t0 = (t0 - ntask) & (tstep - 1);
+    }
+}
+
 // Single-width units (every group of the matrix at width index W, items in
 // (column, row) order, n = rows x cols of them): warp task k covers items
 // SPAN k .. SPAN k + SPAN - 1 (64 at one bit, two per lane; 32 otherwise),
@@ -814,13 +887,16 @@ __device__ __forceinline__ void team_flush(const float* slots, const LayoutView&
 }
 
 // NX activation vectors x (NX x K, row-major) and outputs y (NX x N). SW: the
-// matrix has a single width (L.single_w >= 0; see consume_single).
-template <int NX, int MODE, bool SW = false>
-__global__ void __launch_bounds__(G1_THREADS, 1) gemv1_kernel(LayoutView L, const uint16_t* __restrict__ x,
+// matrix has a single width (L.single_w >= 0; see consume_single). View: the
+// layout, or a wide view of it.
+template <int NX, int MODE, bool SW = false, class View = LayoutView>
+__global__ void __launch_bounds__(G1_THREADS, 1) gemv1_kernel(View V, const uint16_t* __restrict__ x,
                                                               float* __restrict__ y, int dep,
                                                               uint16_t* __restrict__ h,
                                                               const float* __restrict__ gu) {
     static_assert(MODE == MODE_PLAIN || NX == 1, "the SwiGLU forms take one activation vector");
+    constexpr bool WIDE = std::is_same<View, WideView>::value;
+    const LayoutView& L = layout_of(V);
     constexpr int NSTAGE = Geo<NX>::nstage;
     static_assert(NSTAGE % NCOPY == 0, "each stage belongs to one copier");
     // each team flushes its own last unit (the copiers would add a hand-off
@@ -863,7 +939,10 @@ __global__ void __launch_bounds__(G1_THREADS, 1) gemv1_kernel(LayoutView L, cons
     __syncthreads();
     if (tid == 0) {
         const int first = n_units < NSTAGE ? n_units : NSTAGE;
-        for (int j = 0; j < first; ++j) issue_unit_g1<SW>(L, u_begin + j, stage0 + j * STAGE_BYTES, full0 + 8 * j);
+        for (int j = 0; j < first; ++j) {
+            if constexpr (WIDE) issue_wide(V, u_begin + j, stage0 + j * STAGE_BYTES, full0 + 8 * j);
+            else issue_unit_g1<SW>(L, u_begin + j, stage0 + j * STAGE_BYTES, full0 + 8 * j);
+        }
     }
     // Weights never depend on earlier work in the stream, so the first copies
     // are in flight before this grid waits for its predecessor (programmatic
@@ -982,8 +1061,10 @@ __global__ void __launch_bounds__(G1_THREADS, 1) gemv1_kernel(LayoutView L, cons
                     }
                 }
                 __syncwarp();
-                if (j + NSTAGE < n_units && lane == 0)
-                    issue_unit_g1<SW>(L, u_begin + j + NSTAGE, stage0 + st * STAGE_BYTES, full0 + 8 * st);
+                if (j + NSTAGE < n_units && lane == 0) {
+                    if constexpr (WIDE) issue_wide(V, u_begin + j + NSTAGE, stage0 + st * STAGE_BYTES, full0 + 8 * st);
+                    else issue_unit_g1<SW>(L, u_begin + j + NSTAGE, stage0 + st * STAGE_BYTES, full0 + 8 * st);
+                }
                 jdone = j;
                 if (MODE == MODE_SWIGLU_EPI && L.S > 1) {
                     // SwiGLU: count this unit's slab, then act on the previous unit's count
@@ -1044,6 +1125,8 @@ __global__ void __launch_bounds__(G1_THREADS, 1) gemv1_kernel(LayoutView L, cons
                 if constexpr (SW)
                     consume_single<NX>(T, stage0 + st * STAGE_BYTES, smem_u32(T.slots[st][0]), t0, tw, lane,
                                        min(RB, (int)(L.N - (int64_t)rbj * RB)), L.single_w);
+                else if constexpr (WIDE)
+                    consume_wide<NX>(T, V, sj, stage0 + st * STAGE_BYTES, smem_u32(T.slots[st][0]), t0, tw, lane);
                 else
                     consume_unit<NX>(T, stage0 + st * STAGE_BYTES, smem_u32(T.slots[st][0]), t0, tw, lane);
                 __syncwarp();
@@ -1491,19 +1574,15 @@ cudaError_t launch_gemv1_unit(const LayoutView& L, const uint16_t* x, float* y, 
     return cudaGetLastError();
 }
 
-template <int NX, int MODE = MODE_PLAIN, bool SW = false>
-cudaError_t launch_gemv1(const LayoutView& L, const uint16_t* x, float* y, cudaStream_t s, int dep,
-                         uint16_t* h = nullptr, const float* gu = nullptr) {
+template <int NX, int MODE, bool SW, class View>
+cudaError_t launch_gemv1_persistent(const View& V, int units, const uint16_t* x, float* y, cudaStream_t s, int dep,
+                                    uint16_t* h, const float* gu) {
     static LaunchPrep prep;
     int sms = 0;
-    cudaError_t e = prep.get(gemv1_kernel<NX, MODE, SW>, gemv1_smem<NX>(), &sms);
+    cudaError_t e = prep.get(gemv1_kernel<NX, MODE, SW, View>, gemv1_smem<NX>(), &sms);
     if (e != cudaSuccess) return e;
-    if constexpr (NX == 1) {
-        if (runs_unit_per_block(L, sms)) return launch_gemv1_unit<MODE, SW>(L, x, y, s, dep, h, gu);
-    }
-    const int grid = L.units < sms ? L.units : sms;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = dim3(units < sms ? units : sms);
     cfg.blockDim = dim3(G1_THREADS);
     cfg.dynamicSmemBytes = gemv1_smem<NX>();
     cfg.stream = s;
@@ -1512,9 +1591,25 @@ cudaError_t launch_gemv1(const LayoutView& L, const uint16_t* x, float* y, cudaS
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, gemv1_kernel<NX, MODE, SW>, L, x, y, dep, h, gu);
+    e = cudaLaunchKernelEx(&cfg, gemv1_kernel<NX, MODE, SW, View>, V, x, y, dep, h, gu);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
+}
+
+template <int NX, int MODE = MODE_PLAIN, bool SW = false>
+cudaError_t launch_gemv1(const LayoutView& L, const uint16_t* x, float* y, cudaStream_t s, int dep,
+                         uint16_t* h = nullptr, const float* gu = nullptr) {
+    static LaunchPrep prep;
+    int sms = 0;
+    const cudaError_t e = prep.get(gemv1_kernel<NX, MODE, SW>, gemv1_smem<NX>(), &sms);
+    if (e != cudaSuccess) return e;
+    if constexpr (NX == 1) {
+        if (runs_unit_per_block(L, sms)) return launch_gemv1_unit<MODE, SW>(L, x, y, s, dep, h, gu);
+    } else {
+        const WideView V = wide_view(L, sms);
+        if (V.sub > 1) return launch_gemv1_persistent<NX, MODE, SW>(V, V.L.units, x, y, s, dep, h, gu);
+    }
+    return launch_gemv1_persistent<NX, MODE, SW>(L, L.units, x, y, s, dep, h, gu);
 }
 
 }  // namespace

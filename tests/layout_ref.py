@@ -96,3 +96,18 @@ def check(layout, widths):
 def runs_unit_per_block(widths, c, s, units):
     n, g = widths.shape
     return unit_neighbours(g) and unit_plan_fits(c, s, units, n * g, sm_count())
+
+
+def pair_view(widths, c):
+    """(columns per slab, slabs, units) as the two-row table kernel takes a layout of c columns
+    per slab: several slabs as one while there are at least half as many units as SMs and the
+    slabs' blobs fit one stage."""
+    n, g = widths.shape
+    nrb, wide = -(-n // RB), 16
+    while wide > 1 and (wide > g or 2 * nrb * -(-g // wide) < sm_count()):
+        wide //= 2
+    sub, blob = wide // c, 16 * max(unit_sizes(widths, c))
+    while sub > 1 and sub * blob > MAX_BLOB:
+        sub //= 2
+    wide = c * max(sub, 1)
+    return wide, -(-g // wide), nrb * -(-g // wide)
