@@ -23,14 +23,14 @@
 //   Levels and activations are exact and their products accumulate in fp32;
 //   a group whose codes all sit at the zero level gives exactly 0.
 //
-// Bound: instruction issue and its latencies (56% issue, ALU pipe, which runs
-// logic and shifts at half rate, 42% busy, tensor pipe 17%). Per 32 groups of
-// the main mix and 8 rows a warp issues 259 instructions, where fp16 denormal
-// levels, clamped item indexes and per-(row, column) slots took 375. Per
-// product in a graph of dependent products, before -> now: 14336 x 4096 main
-// 18.6 -> 12.6 us at 8 rows and 34.7 -> 17.6 at 16; 16384^2 all 1 bit 59 -> 42
-// and 97 -> 63, all 2 bits 71 -> 46 and 106 -> 64, all 4 bits 72 -> 58 and 121
-// -> 83, all 8 bits 98 -> 97 and 170 -> 136. The error against 64 bits fell
+// Bound: instruction issue and its latencies (8192^2 main at 8 rows: 51% issue,
+// ALU pipe, which runs logic and shifts at half rate, 37% busy, tensor pipe
+// 15%; 16384 x 8192: 55% issue). Per 32 groups of the main mix and 8 rows a warp
+// issues 268 instructions, where fp16 denormal levels, clamped item indexes and
+// per-(row, column) slots took 375. Per product in a graph of dependent
+// products, before -> now: 14336 x 4096 main 18.6 -> 12.5 us at 8 rows and 34.7
+// -> 17.0 at 16; 16384^2 all 1 bit 59 -> 42 and 97 -> 60, all 2 bits 71 -> 46 and
+// 106 -> 63, all 4 bits 72 -> 57 and 121 -> 80, all 8 bits 98 -> 95 and 170 -> 134. The error against 64 bits fell
 // from 5e-6 to 1e-7 of the result's norm: denormal operands lose their
 // alignment in the tensor core's sums, normal bf16 ones do not.
 //
